@@ -56,8 +56,9 @@ struct Smem {
     const float *tab;
     PlanDev *plans;
     WarpState *ws;
-    unsigned long long *cnt;     // [CNT_N]
-    unsigned long long *ledger;  // [n_plans][3]: incident, escaped, rest
+    unsigned int *wcnt;          // [MAX_WARPS][CNT_N] event counters, a row per warp
+    unsigned long long *cnt;     // [CNT_N] cycle profile (64-bit)
+    unsigned int *ledger;        // [n_plans][3][2]: incident, escaped, rest; low and high words
 };
 
 __device__ __forceinline__ float interp(const float *t, float x) {
@@ -165,10 +166,24 @@ __device__ __forceinline__ void deposit_aggregated(const PlanDev &P, uint32_t hi
 }
 
 __device__ __forceinline__ void ledger_add(const Smem &S, uint32_t plan, int which, uint32_t e) {
-    if (e) atomicAdd(&S.ledger[plan * 3 + which], (unsigned long long)e);
+    unsigned int *l = &S.ledger[(plan * 3 + which) * 2];
+    if (atomicAdd(l, e) + e < e) atomicAdd(l + 1, 1u);  // the low word wrapped: carry
 }
 
-__device__ __forceinline__ void count(const Smem &S, int which) { atomicAdd(&S.cnt[which], 1ull); }
+// A warp's event counter: at most 128 increments an iteration (three flights of
+// 32 lanes, or the records a spill moves) and at most 2^24 iterations a launch,
+// so 32 bits hold it.  Counters and ledgers are 32-bit words because shared
+// memory adds 32 bits in one instruction, without a result to wait for, while
+// a 64-bit shared add is a compare-and-swap loop: its lanes retry one after
+// another, and so did the 32 warps of the CTA on the counter they shared.
+// With a row of counters per warp, and ledgers as a low word with a carry, the
+// 15 MeV beams on 128^3 water take 2.11 ms (1e6 electrons) and 4.48 ms (4e6
+// photons) of transport, 2.38 and 5.33 before; the 2 MeV pencil of 1e5
+// photons 0.134 ms, 0.192 before.
+__device__ __forceinline__ unsigned int *counter(const Smem &S, int w, int which) {
+    return &S.wcnt[w * CNT_N + which];
+}
+__device__ __forceinline__ void count(const Smem &S, int w, int which) { atomicAdd(counter(S, w, which), 1u); }
 
 // Rotate (ux, uy, uz) by polar angle (cos c, sin s) and azimuth (cos cp, sin sp).
 __device__ __forceinline__ void rotate(float &ux, float &uy, float &uz, float c, float s, float cp,
@@ -204,7 +219,7 @@ __device__ __forceinline__ void push(const TransportArgs &A, const Smem &S, int 
     r->a = make_float4(x, y, z, ux);
     r->b = make_float4(uy, uz, __uint_as_float(E), __uint_as_float(parent.hist));
     r->c = make_uint4(lo, hi, 0u, parent.plan);
-    count(S, type == 0 ? CNT_PHOTONS : CNT_ELECTRONS);
+    count(S, w, type == 0 ? CNT_PHOTONS : CNT_ELECTRONS);
 }
 
 // An electron set in motion by a photon: pushed for transport, or, in the
@@ -417,7 +432,7 @@ __device__ __forceinline__ uint32_t make_primary(Lane &p, const PlanDev &P, uint
 // by the partial attenuation coefficients of the voxel's material).
 __device__ __forceinline__ bool photon_flight(const TransportArgs &A, const Smem &S, Lane &p, float xp,
                                               float mu_hat, uint32_t &idx_out, uint32_t &rz, int &m_out,
-                                              float &rho_out, float &mu_out) {
+                                              float &rho_out, float &mu_out, int w) {
     const PlanDev &P = S.plans[p.plan];
     const Phys &ph = A.phys;
     const uint4 r = draw4(p, P);
@@ -440,7 +455,7 @@ __device__ __forceinline__ bool photon_flight(const TransportArgs &A, const Smem
     float mu = rho * interp(tp, xp);
     if (!pair_open) mu = rho * (interp(tp + G, xp) + interp(tp + 2 * G, xp));
     if (u01(r.y) * mu_hat > mu) return false;  // fictitious: direction and energy unchanged
-    count(S, CNT_PH_REAL);
+    count(S, w, CNT_PH_REAL);
     idx_out = idx;
     rz = r.z;
     m_out = m;
@@ -463,12 +478,12 @@ __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Sm
     const float E = (float)p.E * kQf;
     if (q < muC) {
         // Compton scattering on a free electron (Klein-Nishina).
-        count(S, CNT_COMPTON);
+        count(S, w, CNT_COMPTON);
         float c;
         uint32_t w4;
         unsigned capped = 0;
         const float eps = sample_kn(p, P, E / kMC2f, &c, &w4, &capped);
-        if (capped) atomicAdd(&S.cnt[CNT_SAMPLER_CAP], 1ull);
+        if (capped) count(S, w, CNT_SAMPLER_CAP);
         float sp, cp;
         __sincosf(kTWO_PIf * u01(w4), &sp, &cp);
         const float sn = sqrtf(fmaxf(0.0f, (1.0f - c) * (1.0f + c)));
@@ -495,12 +510,12 @@ __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Sm
         }
     } else if (q < muC + mupe || !pair_open) {
         // Photoelectric: one K-shell electron carrying all of E (no binding).
-        count(S, CNT_PHOTO);
+        count(S, w, CNT_PHOTO);
         if (p.E >= ph.e_abs_q) {
             uint32_t w3;
             unsigned capped = 0;
             const float c = sample_sauter(p, P, E, &w3, &capped);
-            if (capped) atomicAdd(&S.cnt[CNT_SAMPLER_CAP], 1ull);
+            if (capped) count(S, w, CNT_SAMPLER_CAP);
             float sp, cp;
             __sincosf(kTWO_PIf * u01(w3), &sp, &cp);
             const float sn = sqrtf(fmaxf(0.0f, (1.0f - c) * (1.0f + c)));
@@ -514,7 +529,7 @@ __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Sm
     } else {
         // Pair production without positrons: two electrons share E - 2mc^2
         // uniformly, the rest energy goes to its own ledger.
-        count(S, CNT_PAIR);
+        count(S, w, CNT_PAIR);
         const uint32_t tt = p.E - ph.two_mc2_q;
         ledger_add(S, p.plan, 2, ph.two_mc2_q);
         const uint4 r2 = draw4(p, P);
@@ -662,17 +677,17 @@ __device__ __forceinline__ void hard_event(const TransportArgs &A, const Smem &S
     const float sm = T1 > 2.0f * ph.t_c ? fmaxf(rho1 * interp(t1 + G, xe1) - sb, 0.0f) : 0.0f;
     const float sig = sm + sb;
     if (u01(r2.x) * sig_hat >= sig) {
-        count(S, CNT_HARD_FICT);
+        count(S, w, CNT_HARD_FICT);
         return;
     }
-    count(S, CNT_HARD_REAL);
+    count(S, w, CNT_HARD_REAL);
     if (u01(r2.y) * sig < sm) {
         // Moller: knock-on and scattered electron, azimuths phi and phi + pi
-        count(S, CNT_MOLLER);
+        count(S, w, CNT_MOLLER);
         uint32_t w3;
         unsigned capped = 0;
         const float eps = sample_moller(p, P, T1, ph.t_c, &w3, &capped);
-        if (capped) atomicAdd(&S.cnt[CNT_SAMPLER_CAP], 1ull);
+        if (capped) count(S, w, CNT_SAMPLER_CAP);
         const uint32_t tk = min(e1, __float2uint_rn(eps * (float)e1));
         const uint32_t tp = e1 - tk;
         const float tkf = (float)tk * kQf, tpf = (float)tp * kQf;
@@ -690,12 +705,12 @@ __device__ __forceinline__ void hard_event(const TransportArgs &A, const Smem &S
         p.E = tp;
     } else {
         // bremsstrahlung: electron direction kept, photon at theta = mc^2/E
-        count(S, CNT_BREM);
+        count(S, w, CNT_BREM);
         uint32_t w3;
         unsigned capped = 0;
         const float k = sample_brem(p, P, T1, ph.k_c, S.tab[TAB_BREM + 2 * m1], S.tab[TAB_BREM + 2 * m1 + 1], &w3,
                                     &capped);
-        if (capped) atomicAdd(&S.cnt[CNT_SAMPLER_CAP], 1ull);
+        if (capped) count(S, w, CNT_SAMPLER_CAP);
         const uint32_t kq = min(e1, __float2uint_rn(k * kInvQf));
         const float th = __fdividef(kMC2f, T1 + kMC2f);
         float st, ct, sp, cp;
@@ -739,6 +754,7 @@ struct CtaFlags {
 // mbarrier and the source flags (fixed size, rounded up to 128 bytes), then the
 // tables staged by the bulk copy.
 constexpr size_t SMEM_FIXED = (sizeof(PlanDev) * GPUMCD_MAX_PLANS_PER_RUN + sizeof(WarpState) * MAX_WARPS +
+                               sizeof(unsigned int) * MAX_WARPS * CNT_N +
                                sizeof(unsigned long long) * (CNT_N + 3 * GPUMCD_MAX_PLANS_PER_RUN + 1) +
                                sizeof(CtaFlags) + 127) / 128 * 128;
 
@@ -758,10 +774,10 @@ __device__ void spill_to_queue(const TransportArgs &A, const Smem &S, int gw, in
     if (lane == 0) {
         if (base + n > A.out[t].capacity) {
             atomicExch(A.error, GPUMCD_ERR_QUEUE_OVERFLOW);
-            atomicAdd(&S.cnt[CNT_OVERFLOW], 1ull);
+            count(S, w, CNT_OVERFLOW);
         }
         S.ws[w].stk[t] = top - n;
-        atomicAdd(&S.cnt[CNT_SPILLS], (unsigned long long)n);
+        atomicAdd(counter(S, w, CNT_SPILLS), n);
     }
     __syncwarp();
 }
@@ -877,7 +893,7 @@ __device__ int refill(const TransportArgs &A, const Smem &S, CtaFlags &F, Lane &
         if (lane == 0) {
             ws.p_lo[t] = lo + take;
             ws.p_hi[t] = hi;
-            atomicAdd(&S.cnt[t == 0 ? CNT_PHOTONS : CNT_ELECTRONS], (unsigned long long)take);
+            atomicAdd(counter(S, w, t == 0 ? CNT_PHOTONS : CNT_ELECTRONS), take);
         }
         __syncwarp();
         empty = __ballot_sync(FULL, !p.act);
@@ -937,7 +953,7 @@ __device__ __forceinline__ void hard_pass(const TransportArgs &A, const Smem &S,
     if (lane == 0) {
         S.ws[w].stk[1] = base + __popc(actm);
         S.ws[w].hc = hc - take;
-        atomicAdd(&S.cnt[CNT_HARD_PASSES], 1ull);
+        count(S, w, CNT_HARD_PASSES);
     }
     __syncwarp();
     // headroom for the events' secondaries (at most one per lane per type)
@@ -969,7 +985,8 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
     extern __shared__ __align__(128) unsigned char smem_raw[];
     PlanDev *plans = (PlanDev *)smem_raw;
     WarpState *ws = (WarpState *)(plans + GPUMCD_MAX_PLANS_PER_RUN);
-    unsigned long long *cnt = (unsigned long long *)(ws + MAX_WARPS);
+    unsigned int *wcnt = (unsigned int *)(ws + MAX_WARPS);
+    unsigned long long *cnt = (unsigned long long *)(wcnt + MAX_WARPS * CNT_N);
     unsigned long long *ledger = cnt + CNT_N;
     unsigned long long *mbar = ledger + 3 * GPUMCD_MAX_PLANS_PER_RUN;
     CtaFlags *flags = (CtaFlags *)(mbar + 1);
@@ -1001,6 +1018,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
         ws[i].p_lo[0] = ws[i].p_hi[0] = ws[i].p_lo[1] = ws[i].p_hi[1] = 0;
         ws[i].q_lo[0] = ws[i].q_hi[0] = ws[i].q_lo[1] = ws[i].q_hi[1] = 0;
     }
+    for (int i = tid; i < MAX_WARPS * CNT_N; i += blockDim.x) wcnt[i] = 0u;
     for (int i = tid; i < CNT_N + 3 * GPUMCD_MAX_PLANS_PER_RUN; i += blockDim.x) cnt[i] = 0;
     if (tid < 2) {
         flags->in_done[tid] = A.in_count[tid] == 0;
@@ -1021,7 +1039,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
         if (tid == 0) atomicExch(A.error, GPUMCD_ERR_TIMEOUT);
         return;
     }
-    const Smem S{tab, plans, ws, cnt, ledger};
+    const Smem S{tab, plans, ws, wcnt, cnt, (unsigned int *)ledger};
     CtaFlags &F = *flags;
 
     Lane p;
@@ -1124,16 +1142,17 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
                 const bool fly = p.act && !real;
                 const unsigned flym = __ballot_sync(FULL, fly);
                 if (flym == 0u) break;
-                if (lane == 0) atomicAdd(&S.cnt[CNT_PH_EVENTS], (unsigned long long)__popc(flym));
-                if (fly) real = photon_flight(A, S, p, xp, mu_hat, pidx, prz, rm, rrho, rmu);
+                if (fly) {
+                    count(S, w, CNT_PH_EVENTS);
+                    real = photon_flight(A, S, p, xp, mu_hat, pidx, prz, rm, rrho, rmu, w);
+                }
             }
             if (real) photon_interact<KERMA>(A, S, p, pidx, prz, xp, rm, rrho, rmu, gw, w);
         } else {
             uint32_t dep_idx = 0, dep_e = 0;
             bool stepped = false;
             if (p.act) stepped = electron_step(A, S, p, gw, w, dep_idx, dep_e);
-            const unsigned sm = __ballot_sync(FULL, stepped);
-            if (lane == 0) atomicAdd(&S.cnt[CNT_E_STEPS], (unsigned long long)__popc(sm));
+            if (stepped) count(S, w, CNT_E_STEPS);
             const PlanDev &P = S.plans[p.plan];
             if (agg)
                 deposit_aggregated(P, p.hist, dep_idx, dep_e);
@@ -1150,8 +1169,11 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
         }
     }
     __syncthreads();
-    for (int i = tid; i < CNT_N; i += blockDim.x)
-        if (cnt[i]) atomicAdd(&A.counters[i], cnt[i]);
+    for (int i = tid; i < CNT_N; i += blockDim.x) {
+        unsigned long long n = cnt[i];
+        for (int k = 0; k < MAX_WARPS; ++k) n += wcnt[k * CNT_N + i];
+        if (n) atomicAdd(&A.counters[i], n);
+    }
     for (int i = tid; i < 3 * A.n_plans; i += blockDim.x)
         if (ledger[i]) atomicAdd(&plans[i / 3].ledger[i % 3], ledger[i]);
 }
