@@ -92,7 +92,7 @@ struct __align__(16) HardRec {
     uint32_t idx;
     uint32_t pad[2];
 };
-constexpr unsigned HARD_CAP = 64;  // per warp: a pass starts at 32, one step adds at most 32
+constexpr unsigned HARD_CAP = 64;  // per warp: a pass starts at 32, the steps between refills add at most 32
 
 // One plan inside a launch (copied to shared memory by the transport kernel).
 struct __align__(16) PlanDev {
