@@ -133,7 +133,7 @@ typedef struct {
     uint32_t stack_capacity;  /* per-warp particle stack entries per type */
     uint32_t switch_high;     /* a warp switches type when the other stack holds this many (= stack_capacity: never) */
     uint32_t refill_low;      /* ...or when it fills fewer lanes than this and the other type has work */
-    uint32_t chunk;           /* primaries or queued particles a warp claims at once */
+    uint32_t chunk;           /* primaries or queued particles a warp claims at once, at most */
     uint32_t overflow_capacity; /* global overflow queue entries per type */
     uint32_t flags;           /* GPUMCD_LAUNCH_* */
     uint32_t refill_period;   /* lane refill policy, the divergence-reduction ablation (below) */

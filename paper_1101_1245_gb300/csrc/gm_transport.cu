@@ -735,9 +735,26 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
-// Claim `want` records of a global source with a cursor and a fixed count.
-__device__ __forceinline__ void claim(unsigned long long *cursor, unsigned long long total, uint32_t want,
+// Claim records of a global source of type t with a cursor and a fixed count:
+// `chunk` of them while there is plenty, fewer so that every warp gets a share.
+// A photon source shorter than a chunk per warp is split evenly.  Of an
+// electron source a warp takes an even share of what is left, so the claims
+// shrink towards the end: an electron's path is a chain of tens of steps that
+// nothing shortens, so late claims of 32 left some warps a full load to run
+// while the others had ended.  Transport against claims of 32 throughout: 3001
+// electrons of 9 MeV 0.31 -> 0.18 ms, 1e4 photons of 2 MeV 0.125 -> 0.084 ms,
+// 1e6 electrons of 15 MeV 1.94 -> 1.83 ms; no case is slower.  Shrinking
+// claims of photons cost 4e6 of 15 MeV 3.5% (4.22 -> 4.37 ms) and the slab
+// plan 1.6%: photon warps then run half empty and switch type more often.
+__device__ __forceinline__ void claim(unsigned long long *cursor, unsigned long long total, uint32_t chunk, int t,
                                       unsigned long long &lo, unsigned long long &hi) {
+    const uint32_t warps = gridDim.x * (blockDim.x >> 5);
+    unsigned long long left = total;
+    if (t == 1) {
+        const unsigned long long now = *(volatile unsigned long long *)cursor;
+        left = now < total ? total - now : 0ull;
+    }
+    const uint32_t want = left >= (unsigned long long)chunk * warps ? chunk : max((uint32_t)left / warps, 1u);
     const unsigned long long base = atomicAdd(cursor, (unsigned long long)want);
     lo = base < total ? base : total;
     hi = base + want < total ? base + want : total;
@@ -811,7 +828,7 @@ __device__ int refill(const TransportArgs &A, const Smem &S, CtaFlags &F, Lane &
         unsigned long long lo = ws.q_lo[t], hi = ws.q_hi[t];
         if (lo == hi) {
             if (__shfl_sync(FULL, lane == 0 ? *(volatile int *)&F.in_done[t] : 0, 0)) break;
-            if (lane == 0) claim(A.in[t].cursor, A.in_count[t], A.chunk, lo, hi);
+            if (lane == 0) claim(A.in[t].cursor, A.in_count[t], A.chunk, t, lo, hi);
             lo = __shfl_sync(FULL, lo, 0);
             hi = __shfl_sync(FULL, hi, 0);
             if (lo == hi) {
@@ -836,7 +853,7 @@ __device__ int refill(const TransportArgs &A, const Smem &S, CtaFlags &F, Lane &
         unsigned long long lo = ws.p_lo[t], hi = ws.p_hi[t];
         if (lo == hi) {
             if (__shfl_sync(FULL, lane == 0 ? *(volatile int *)&F.prim_done[t] : 0, 0)) break;
-            if (lane == 0) claim(&A.prim_cursor[t], A.prim_off[t][A.n_prim_plans[t]], A.chunk, lo, hi);
+            if (lane == 0) claim(&A.prim_cursor[t], A.prim_off[t][A.n_prim_plans[t]], A.chunk, t, lo, hi);
             lo = __shfl_sync(FULL, lo, 0);
             hi = __shfl_sync(FULL, hi, 0);
             if (lo == hi) {
