@@ -310,43 +310,46 @@ __device__ float sample_sauter(Lane &p, const PlanDev &P, float T, uint32_t *w3,
     }
 }
 
-// Moller knock-on fraction in [t_c/T, 1/2] (§II.B.1): 1/eps^2 proposal.
-__device__ float sample_moller(Lane &p, const PlanDev &P, float T, float t_c, uint32_t *w3, unsigned *capped) {
-    const float g = T / kMC2f + 1.0f;
-    const float c1 = __fdividef((g - 1.0f) * (g - 1.0f), g * g);
-    const float c2 = __fdividef(2.0f * g - 1.0f, g * g);
-    const float ec = __fdividef(t_c, T);
-    const float bound = 2.0f + 0.25f * c1;
-    for (int it = 0;; ++it) {
-        const uint4 r = draw4(p, P);
-        const float eps = __fdividef(ec, 1.0f - u01(r.x) * (1.0f - 2.0f * ec));
-        const float q = __fdividef(eps, 1.0f - eps);
-        const float f = 1.0f + q * q + c1 * eps * eps - c2 * q;
-        const bool ok = u01(r.y) * bound <= f;
-        if (ok || it >= SAMPLER_CAP) {
-            if (!ok) ++*capped;
-            *w3 = r.z;
-            return eps;
-        }
+// Hard electron event (§II.B.1).  Moller: the knock-on fraction in [thr/T, 1/2]
+// by a 1/eps^2 proposal (thr = t_c).  Bremsstrahlung: the photon energy in
+// [thr, T] by a 1/k proposal (thr = k_c), accepted with the normalised shape
+// (4/3 - 4y/3 + y^2) cA + (1 - y) cB.  One loop serves both, so the lanes of a
+// warp share each proposal's draw (ten Philox rounds, most of a proposal)
+// whichever kind they sample.
+__device__ __forceinline__ float sample_hard(Lane &p, const PlanDev &P, bool moller, float T, float thr, float cA,
+                                             float cB, uint32_t *w3, unsigned *capped) {
+    float v0, v1, v2, v3;  // Moller: thr / T, c1, c2, bound; bremsstrahlung: E, ln(T / thr), cA, cB
+    if (moller) {
+        const float g = T / kMC2f + 1.0f;
+        v0 = __fdividef(thr, T);
+        v1 = __fdividef((g - 1.0f) * (g - 1.0f), g * g);
+        v2 = __fdividef(2.0f * g - 1.0f, g * g);
+        v3 = 2.0f + 0.25f * v1;
+    } else {
+        v0 = T + kMC2f;
+        v1 = __logf(__fdividef(T, thr));
+        v2 = cA;
+        v3 = cB;
     }
-}
-
-// Bremsstrahlung photon energy in [k_c, T] (§II.B.1): 1/k proposal, accepted
-// with the normalised shape (4/3 - 4y/3 + y^2) cA + (1 - y) c1.
-__device__ float sample_brem(Lane &p, const PlanDev &P, float T, float k_c, float cA, float c1,
-                             uint32_t *w3, unsigned *capped) {
-    const float E = T + kMC2f;
-    const float lr = __logf(__fdividef(T, k_c));
     for (int it = 0;; ++it) {
         const uint4 r = draw4(p, P);
-        const float k = k_c * __expf(u01(r.x) * lr);
-        const float y = __fdividef(k, E);
-        const float gy = fmaf(y, y - 4.0f / 3.0f, 4.0f / 3.0f) * cA + (1.0f - y) * c1;
-        const bool ok = u01(r.y) <= gy;
+        float x;
+        bool ok;
+        if (moller) {
+            x = __fdividef(v0, 1.0f - u01(r.x) * (1.0f - 2.0f * v0));
+            const float q = __fdividef(x, 1.0f - x);
+            const float f = 1.0f + q * q + v1 * x * x - v2 * q;
+            ok = u01(r.y) * v3 <= f;
+        } else {
+            x = thr * __expf(u01(r.x) * v1);
+            const float y = __fdividef(x, v0);
+            const float gy = fmaf(y, y - 4.0f / 3.0f, 4.0f / 3.0f) * v2 + (1.0f - y) * v3;
+            ok = u01(r.y) <= gy;
+        }
         if (ok || it >= SAMPLER_CAP) {
             if (!ok) ++*capped;
             *w3 = r.z;
-            return k;
+            return x;
         }
     }
 }
@@ -681,49 +684,43 @@ __device__ __forceinline__ void hard_event(const TransportArgs &A, const Smem &S
         return;
     }
     count(S, w, CNT_HARD_REAL);
-    if (u01(r2.y) * sig < sm) {
-        // Moller: knock-on and scattered electron, azimuths phi and phi + pi
-        count(S, w, CNT_MOLLER);
-        uint32_t w3;
-        unsigned capped = 0;
-        const float eps = sample_moller(p, P, T1, ph.t_c, &w3, &capped);
-        if (capped) count(S, w, CNT_SAMPLER_CAP);
-        const uint32_t tk = min(e1, __float2uint_rn(eps * (float)e1));
-        const uint32_t tp = e1 - tk;
-        const float tkf = (float)tk * kQf, tpf = (float)tp * kQf;
-        const float ck = sqrtf(fminf(1.0f, __fdividef(tkf * (T1 + 2.0f * kMC2f), T1 * (tkf + 2.0f * kMC2f))));
-        const float cpp = sqrtf(fminf(1.0f, __fdividef(tpf * (T1 + 2.0f * kMC2f), T1 * (tpf + 2.0f * kMC2f))));
-        float sp, cp;
-        __sincosf(kTWO_PIf * u01(w3), &sp, &cp);
-        float vx = p.ux, vy = p.uy, vz = p.uz;
-        rotate(vx, vy, vz, ck, sqrtf(fmaxf(0.f, 1.f - ck * ck)), cp, sp);
-        rotate(p.ux, p.uy, p.uz, cpp, sqrtf(fmaxf(0.f, 1.f - cpp * cpp)), -cp, -sp);
-        if (tk >= ph.e_abs_q)
-            push(A, S, gw, w, 1, p.x, p.y, p.z, vx, vy, vz, tk, p, 0);
-        else
-            deposit(P, p.hist, idx1, tk);
-        p.E = tp;
+    const bool moller = u01(r2.y) * sig < sm;
+    count(S, w, moller ? CNT_MOLLER : CNT_BREM);
+    // The two kinds share the proposals' draws, the azimuth, the rotation and
+    // the push of the new particle.  As two branches, each ran its own copy
+    // with its part of the lanes (about two thirds Moller): 15 MeV electrons
+    // on 128^3 water took 1.85 ms of transport, 1.77 this way, photons 4.19
+    // and 4.09.
+    uint32_t w3;
+    unsigned capped = 0;
+    const float x = sample_hard(p, P, moller, T1, moller ? ph.t_c : ph.k_c, S.tab[TAB_BREM + 2 * m1],
+                                S.tab[TAB_BREM + 2 * m1 + 1], &w3, &capped);
+    if (capped) count(S, w, CNT_SAMPLER_CAP);
+    uint32_t e2;
+    float c, sn, c2 = 1.0f;
+    if (moller) {
+        // knock-on and scattered electron, azimuths phi and phi + pi
+        e2 = min(e1, __float2uint_rn(x * (float)e1));
+        const uint32_t tp = e1 - e2;
+        const float tkf = (float)e2 * kQf, tpf = (float)tp * kQf;
+        c = sqrtf(fminf(1.0f, __fdividef(tkf * (T1 + 2.0f * kMC2f), T1 * (tkf + 2.0f * kMC2f))));
+        c2 = sqrtf(fminf(1.0f, __fdividef(tpf * (T1 + 2.0f * kMC2f), T1 * (tpf + 2.0f * kMC2f))));
+        sn = sqrtf(fmaxf(0.f, 1.f - c * c));
     } else {
-        // bremsstrahlung: electron direction kept, photon at theta = mc^2/E
-        count(S, w, CNT_BREM);
-        uint32_t w3;
-        unsigned capped = 0;
-        const float k = sample_brem(p, P, T1, ph.k_c, S.tab[TAB_BREM + 2 * m1], S.tab[TAB_BREM + 2 * m1 + 1], &w3,
-                                    &capped);
-        if (capped) count(S, w, CNT_SAMPLER_CAP);
-        const uint32_t kq = min(e1, __float2uint_rn(k * kInvQf));
-        const float th = __fdividef(kMC2f, T1 + kMC2f);
-        float st, ct, sp, cp;
-        __sincosf(th, &st, &ct);
-        __sincosf(kTWO_PIf * u01(w3), &sp, &cp);
-        float vx = p.ux, vy = p.uy, vz = p.uz;
-        rotate(vx, vy, vz, ct, st, cp, sp);
-        if (kq >= ph.p_cut_q)
-            push(A, S, gw, w, 0, p.x, p.y, p.z, vx, vy, vz, kq, p, 0);
-        else
-            deposit(P, p.hist, idx1, kq);
-        p.E = e1 - kq;
+        // electron direction kept, photon at theta = mc^2/E
+        e2 = min(e1, __float2uint_rn(x * kInvQf));
+        __sincosf(__fdividef(kMC2f, T1 + kMC2f), &sn, &c);
     }
+    float sp, cp;
+    __sincosf(kTWO_PIf * u01(w3), &sp, &cp);
+    float vx = p.ux, vy = p.uy, vz = p.uz;
+    rotate(vx, vy, vz, c, sn, cp, sp);
+    if (e2 >= (moller ? ph.e_abs_q : ph.p_cut_q))
+        push(A, S, gw, w, moller ? 1 : 0, p.x, p.y, p.z, vx, vy, vz, e2, p, 0);
+    else
+        deposit(P, p.hist, idx1, e2);
+    if (moller) rotate(p.ux, p.uy, p.uz, c2, sqrtf(fmaxf(0.f, 1.f - c2 * c2)), -cp, -sp);
+    p.E = e1 - e2;
 }
 
 // ---------------------------------------------------------------------------
@@ -1463,9 +1460,9 @@ __global__ void k_debug_sample(const float *tabg, Phys ph, int kind, float p0, i
     } else if (kind == 1) {
         v = sample_sauter(p, P, p0, &wd, &capped);
     } else if (kind == 2) {
-        v = sample_moller(p, P, p0, ph.t_c, &wd, &capped);
+        v = sample_hard(p, P, true, p0, ph.t_c, 0.f, 0.f, &wd, &capped);
     } else if (kind == 3) {
-        v = sample_brem(p, P, p0, ph.k_c, __ldg(tabg + TAB_BREM + 2 * material),
+        v = sample_hard(p, P, false, p0, ph.k_c, __ldg(tabg + TAB_BREM + 2 * material),
                         __ldg(tabg + TAB_BREM + 2 * material + 1), &wd, &capped);
     } else if (kind == 4) {
         // the transport's own ms_mu, given the tables in global memory instead
