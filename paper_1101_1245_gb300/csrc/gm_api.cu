@@ -1102,26 +1102,22 @@ gpumcd_status gpumcd_plan_result(gpumcd_ctx *c, int32_t plan_id, double thr, dou
     Plan &p = it->second;
     const Phantom &ph = c->phantoms.at(p.phantom);
     const uint64_t nvox = ph.nvox;
-    // scratch: [dose | sigma] when the caller passes NULL, then [n_b (64) | dmax | sum | count | esum],
+    // scratch: [dose | sigma] when the caller passes NULL, then [dmax | sum | count | esum],
     // then the s_thr reduction's per-block partials
-    const size_t need = (size_t)nvox * 16 + 64 * 8 + 64 + (size_t)sthr_blocks(nvox, c->n_sm) * 16;
+    const size_t need = (size_t)nvox * 16 + 64 + (size_t)sthr_blocks(nvox, c->n_sm) * 16;
     ST(dev_alloc(c, c->fold_tmp, need));
     double *tdose = (double *)c->fold_tmp.p;
     double *tsig = tdose + nvox;
-    double *nb = tsig + nvox;
-    unsigned long long *red = (unsigned long long *)(nb + 64);
+    unsigned long long *red = (unsigned long long *)(tsig + nvox);
     void *sthr_part = red + 8;
     double *ddose = dose ? dose : tdose;
     double *dsig = sigma ? sigma : tsig;
-    double h_nb[64] = {0};
     const uint64_t N = p.hist_done;
-    // history h belongs to batch h mod W
-    for (uint32_t b = 0; b < p.W; ++b) h_nb[b] = (double)(N / p.W + (b < N % p.W ? 1u : 0u));
     CK(cudaMemsetAsync(red, 0, 64, s));
     const double inv_vol = 1.0 / (ph.voxel[0] * ph.voxel[1] * ph.voxel[2]);
     if (N > 0) {
-        CK(launch_fold((const unsigned long long *)p.tally.p, (const uint32_t *)ph.vox.p, nvox, (int)p.W, h_nb,
-                       (double)N, inv_vol, ddose, dsig, red, red + 3, c->n_sm, s));
+        CK(launch_fold((const unsigned long long *)p.tally.p, (const uint32_t *)ph.vox.p, nvox, (int)p.W, N, inv_vol,
+                       ddose, dsig, red, red + 3, c->n_sm, s));
         CK(launch_sthr(ddose, dsig, nvox, red, thr, (double *)(red + 1), red + 2, sthr_part, c->n_sm, s));
     } else {
         CK(cudaMemsetAsync(ddose, 0, nvox * 8, s));
@@ -1163,13 +1159,10 @@ gpumcd_status gpumcd_plan_result_noalloc(gpumcd_ctx *c, int32_t plan_id, double 
     if (N == 0) return GPUMCD_ERR_STATE;
     ST(set_device(c));
     cudaStream_t s = pick(c, stream);
-    double h_nb[64] = {0};
-    // history h belongs to batch h mod W
-    for (uint32_t b = 0; b < p.W; ++b) h_nb[b] = (double)(N / p.W + (b < N % p.W ? 1u : 0u));
     unsigned long long res[4] = {0, 0, 0, 0}, led[4] = {0, 0, 0, 0};
     const double inv_vol = 1.0 / (ph.voxel[0] * ph.voxel[1] * ph.voxel[2]);
     CK(launch_fold_noalloc(c->device, (const unsigned long long *)p.tally.p, (const uint32_t *)ph.vox.p, ph.nvox,
-                           (int)p.W, h_nb, (double)N, inv_vol, thr, dose, sigma, s, res));
+                           (int)p.W, N, inv_vol, thr, dose, sigma, s, res));
     CK(cudaMemcpyAsync(led, p.ledger.p, sizeof led, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (stats) {

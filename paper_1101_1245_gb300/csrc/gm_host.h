@@ -24,9 +24,10 @@ cudaError_t launch_pack_phantom(const uint8_t *mat, const float *rho, uint64_t n
 cudaError_t launch_majorants(const float *tab, const unsigned int *rho_max_bits, int n_mat, float *maj,
                              cudaStream_t s);
 cudaError_t launch_spectrum(const double *edges, const double *w, int n, float *out, cudaStream_t s);
-cudaError_t launch_fold(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox, int W,
-                        const double *n_b, double n_tot, double inv_vol, double *dose, double *sigma,
-                        unsigned long long *dmax_bits, unsigned long long *dep_sum, int n_sm, cudaStream_t s);
+// Dose and sigma (either may be null) of n_hist histories in W batches, history h in batch h mod W.
+cudaError_t launch_fold(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox, int W, uint64_t n_hist,
+                        double inv_vol, double *dose, double *sigma, unsigned long long *dmax_bits,
+                        unsigned long long *dep_sum, int n_sm, cudaStream_t s);
 // Blocks of the s_thr reduction for nvox voxels: its partials take 16 bytes each.
 int sthr_blocks(uint64_t nvox, int n_sm);
 cudaError_t launch_sthr(const double *dose, const double *sigma, uint64_t nvox,
@@ -35,8 +36,8 @@ cudaError_t launch_sthr(const double *dose, const double *sigma, uint64_t nvox,
 cudaError_t launch_sum_u64(const unsigned long long *a, uint64_t n, unsigned long long *out, int n_sm,
                            cudaStream_t s);
 cudaError_t launch_fold_noalloc(int device, const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
-                                int W, const double *n_b, double n_tot, double inv_vol, double thr, double *dose,
-                                double *sigma, cudaStream_t s, unsigned long long result[4]);
+                                int W, uint64_t n_hist, double inv_vol, double thr, double *dose, double *sigma,
+                                cudaStream_t s, unsigned long long result[4]);
 cudaError_t launch_philox(const uint32_t *ctr, uint2 key, uint64_t n, int curand, uint32_t *out,
                           cudaStream_t s);
 

@@ -2,6 +2,8 @@
 // packing, majorants, spectrum CDF, the dose/uncertainty fold and reductions.
 #include <curand_kernel.h>
 
+#include <cmath>
+
 #include <mutex>
 
 #include "gm_common.cuh"
@@ -314,77 +316,34 @@ __global__ void k_spectrum(const double *edges, const double *w, int n, float *o
 }
 
 // Fold of a plan's batch tallies (GPUMCD §II.D): mean dose per history and
-// the standard error of the mean from the W batch sums S_b (n_b histories
-// each), in FP64:
-//   D = sum_b S_b / N,   var(D) = W / ((W - 1) N^2) sum_b (S_b - n_b D)^2
+// the standard error of the mean from the W batch sums S_b, in FP64:
+//   D = S / N,   var(D) = W / ((W - 1) N^2) sum_b (S_b - n_b D)^2,   S = sum_b S_b
 // (the batch-mean estimator; it reduces to sum (d_b - D)^2 / (W (W - 1)) for
-// equal batches).  The sum over batches is an exact integer; the per-voxel
-// integer sums are also added into the plan's deposited-energy ledger.
-struct FoldArgs {
-    double n_b[64];
+// equal batches).  History h belongs to batch h mod W, so the first N mod W
+// batches hold one history more than the others.  The sum over batches is an
+// exact integer; the per-voxel integer sums are also added into the plan's
+// deposited-energy ledger.
+//
+// GB300 issues two FP64 operations a clock and SM, so a voxel's FP64 work, not
+// its W x 8 bytes, bounded this kernel: about 31 operations a voxel (a
+// division, a square root and conversions among them) held it at 34% of the
+// copy rate.  Now the sums are formed in integers, rounded to FP64 by integer
+// instructions, and the division and square root start from the FP32
+// reciprocal and reciprocal square root and take one third-order step: 12
+// operations a voxel (about 25 with unequal batches, 85 before), none for a
+// voxel without dose, and dose and sigma are as close to the exact values as
+// before or closer.  A result call (fold, s_thr, read-back of the stats) of
+// 256^3 voxels, equal / unequal batches: 16 batches 0.53 / 0.97 ms (1.07 /
+// 3.00 before; the bytes alone take 0.37 at the copy rate), 64 batches 1.49 /
+// 2.36 ms (2.29 / 7.36; 1.32).
+struct FoldConst {
+    double k_dose;   // (q * (MeV/g -> Gy) / (voxel volume * density quantum)) / N
+    double k_sigma;  // ... times sqrt(W / (W - 1)) (unequal batches) or sqrt(1 / (W - 1)) (equal)
+    double inv_n;    // 1 / N
+    double q_n;      // (N div W) / N
+    uint32_t r;      // N mod W: the batches with one history more
 };
 
-// Per-voxel arithmetic of the fold with per-batch history counts n_b: the
-// mean energy per history and the batch-mean variance, scaled to Gy.
-template <int W>
-__device__ __forceinline__ void fold_voxel(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
-                                           uint64_t v, const FoldArgs &fa, double n_tot, double inv_vol,
-                                           double &dv, double &sv, unsigned long long &tot_out) {
-    unsigned long long s[W];
-    unsigned long long tot = 0;
-#pragma unroll
-    for (int b = 0; b < W; ++b) {
-        s[b] = __ldcs(tally + (uint64_t)b * nvox + v);
-        tot += s[b];
-    }
-    const double mean = (double)tot / n_tot;
-    double acc = 0.0;
-#pragma unroll
-    for (int b = 0; b < W; ++b) {
-        const double t = fma(-fa.n_b[b], mean, (double)s[b]);
-        acc = fma(t, t, acc);
-    }
-    const double var = acc * ((double)W / ((double)(W - 1) * n_tot * n_tot));
-    const double rho = (double)(vox[v] >> 4) * (double)kRhoQ;
-    const double scale = kQ * kMeVPerGramToGy * inv_vol / rho;
-    dv = mean * scale;
-    sv = sqrt(var) * scale;
-    tot_out = tot;
-}
-
-template <int W>
-__global__ void k_fold(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
-                       const __grid_constant__ FoldArgs fa, double n_tot, double inv_vol, double *dose,
-                       double *sigma, unsigned long long *dmax_bits, unsigned long long *dep_sum) {
-    double local_max = 0.0;
-    unsigned long long local_sum = 0;
-    for (uint64_t v = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; v < nvox;
-         v += (uint64_t)gridDim.x * blockDim.x) {
-        double dv, sv;
-        unsigned long long tot;
-        fold_voxel<W>(tally, vox, nvox, v, fa, n_tot, inv_vol, dv, sv, tot);
-        if (dose) dose[v] = dv;
-        if (sigma) sigma[v] = sv;
-        local_max = fmax(local_max, dv);
-        local_sum += tot;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        local_max = fmax(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));
-        local_sum += __shfl_xor_sync(0xffffffffu, local_sum, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomicMax(dmax_bits, (unsigned long long)__double_as_longlong(local_max));
-        if (local_sum) atomicAdd(dep_sum, local_sum);
-    }
-}
-
-// The same fold for equal batches (n_b = N / W for every b): the variance
-// numerator is formed exactly in 128-bit integers,
-//   sum_b (S_b - S/W)^2 = (W sum_b S_b^2 - S^2) / W,
-// so only one conversion to FP64 per voxel remains (FP64 is scarce on GB300
-// and the per-batch FP64 work of k_fold bounds it).  A voxel whose sums would
-// not fit 128 bits (sum S_b^2 >= 2^121, far beyond realistic tallies) takes
-// the FP64 two-pass form instead.
 struct U128 {
     unsigned long long lo, hi;
 };
@@ -396,78 +355,185 @@ __device__ __forceinline__ void add_sq(U128 &acc, unsigned long long x) {
     acc.lo = nl;
 }
 
+// v rounded to the nearest double (ties to even), by integer instructions.
 __device__ __forceinline__ double u128_to_double(U128 v) {
-    return (double)v.hi * 18446744073709551616.0 + (double)v.lo;
+    if ((v.hi | v.lo) == 0ull) return 0.0;
+    const int n = __clzll((long long)(v.hi ? v.hi : v.lo));
+    unsigned long long m;  // the leading 64 bits, the rest of the 128 ORed into the last
+    if (v.hi) {
+        m = (v.hi << n) | (v.lo >> 1 >> (63 - n));
+        m |= (v.lo << n) != 0ull ? 1ull : 0ull;
+    } else {
+        m = v.lo << n;
+    }
+    unsigned long long k = m >> 11;
+    const unsigned rest = (unsigned)m & 0x7FFu;
+    k += (rest > 0x400u || (rest == 0x400u && (k & 1ull))) ? 1ull : 0ull;
+    return __longlong_as_double((long long)(((unsigned long long)(1022 + (v.hi ? 127 : 63) - n) << 52) + k));
 }
 
-// FP64 is scarce on GB300, so the per-voxel FP64 work is one division (by
-// the voxel's density code, shared by dose and sigma) and one square root;
-// the other divisors are loop constants whose reciprocals come from the host.
-struct FoldConst {
-    double inv_n;   // 1 / N
-    double c_var;   // 1 / (W^2 (W - 1) n^2), n = N / W
-    double k_dose;  // q * (MeV/g -> Gy) / (voxel volume * density quantum)
-};
+__device__ __forceinline__ double float_to_double(float x) {  // normal x > 0
+    const unsigned b = __float_as_uint(x);
+    return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
+}
 
-// Per-voxel arithmetic of the equal-batch fold.
+// 1 / code for 1 <= code < 2^28: the FP32 reciprocal y has a relative error e
+// below 2^-22, and y (1 + e + e^2) one of e^3.
+__device__ __forceinline__ double rcp_code(uint32_t code) {
+    const int n = __clz((int)code);
+    const uint32_t m = code << n;
+    const double d = __hiloint2double((int)(((uint32_t)(1053 - n) << 20) + (m >> 11)), (int)(m << 21));
+    const double y = float_to_double(__fdividef(1.0f, (float)code));
+    const double e = fma(-d, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+// sqrt(v) for v = 0 or normal v > 0: v = m 4^k with m in [1, 4), y the FP32
+// reciprocal square root of m's leading 24 bits, g = m y and e = 1 - g y
+// (below 2^-20); then sqrt(m) = g (1 - e)^(-1/2) = g + g e (1/2 + 3/8 e) + O(e^3).
+__device__ __forceinline__ double sqrt_fold(double v) {
+    const int hi = __double2hiint(v), lo = __double2loint(v);
+    if (hi <= 0) return 0.0;  // 0, or a rounding's width below
+    const int ex = (hi >> 20) - 1023, odd = ex & 1;
+    const double m = __hiloint2double((hi & 0xFFFFF) | ((1023 + odd) << 20), lo);
+    const float mf = __int_as_float(((127 + odd) << 23) | ((hi & 0xFFFFF) << 3) | (int)((unsigned)lo >> 29));
+    const double y = float_to_double(rsqrtf(mf));
+    const double g = m * y;
+    const double e = fma(-g, y, 1.0);
+    const double s = fma(g * e, fma(e, 0.375, 0.5), g);
+    return __hiloint2double(__double2hiint(s) + (((ex - odd) >> 1) << 20), __double2loint(s));
+}
+
+// The two-pass form in FP64, for sums of squares beyond 128 bits (far beyond
+// realistic tallies): sum_b (S_b - n_b D)^2.
+__device__ __noinline__ double two_pass(const unsigned long long *tally, uint64_t nvox, int W, uint64_t v, double tot,
+                                        const FoldConst &fc) {
+    const double a0 = tot * fc.q_n, a1 = fma(tot, fc.inv_n, a0);
+    double acc = 0.0;
+    for (int b = 0; b < W; ++b) {
+        const double t = (double)tally[(uint64_t)b * nvox + v] - (b < (int)fc.r ? a1 : a0);
+        acc = fma(t, t, acc);
+    }
+    return acc;
+}
+
+// Equal batches (n_b = N / W for every b): the variance numerator is formed
+// exactly in 128-bit integers,
+//   W sum_b (S_b - S/W)^2 = W sum_b S_b^2 - S^2.
 template <int W>
 __device__ __forceinline__ void fold_voxel_equal(const unsigned long long *tally, const uint32_t *vox,
                                                  uint64_t nvox, uint64_t v, const FoldConst &fc, double &dv,
                                                  double &sv, unsigned long long &tot_out) {
-    unsigned long long s[W];
+    constexpr int K = W < 16 ? W : 16;  // loads in flight
     unsigned long long tot = 0;
     U128 sq{0ull, 0ull};
+#pragma unroll
+    for (int b0 = 0; b0 < W; b0 += K) {
+        unsigned long long s[K];
+#pragma unroll
+        for (int b = 0; b < K; ++b) s[b] = __ldcs(tally + (uint64_t)(b0 + b) * nvox + v);
+#pragma unroll
+        for (int b = 0; b < K; ++b) {
+            tot += s[b];
+            add_sq(sq, s[b]);
+        }
+    }
+    const uint32_t code = vox[v] >> 4;
+    tot_out = tot;
+    dv = sv = 0.0;
+    if (tot == 0ull) return;
+    const double td = u128_to_double(U128{tot, 0ull});
+    double num;  // W sum_b (S_b - S/W)^2, in quanta^2
+    if (sq.hi < (1ull << 57)) {
+        const U128 ws{sq.lo * (unsigned long long)W, sq.hi * (unsigned long long)W + __umul64hi(sq.lo, (unsigned long long)W)};
+        const U128 t2{tot * tot, __umul64hi(tot, tot)};
+        num = u128_to_double(U128{ws.lo - t2.lo, ws.hi - t2.hi - (ws.lo < t2.lo ? 1ull : 0ull)});
+    } else {
+        num = two_pass(tally, nvox, W, v, td, fc) * (double)W;
+    }
+    const double y = rcp_code(code);
+    dv = td * fc.k_dose * y;
+    sv = sqrt_fold(num) * fc.k_sigma * y;
+}
+
+// Any batch counts: with i the integer nearest (N div W) D and u_b = S_b - i,
+// S_b - n_b D = u_b - f, where f = (N div W) D - i, plus D for the first r
+// batches; so
+//   sum_b (S_b - n_b D)^2 = sum u_b^2 + f1 (r f1 - 2 sum_{b<r} u_b) + f0 ((W-r) f0 - 2 sum_{b>=r} u_b),
+// whose sums are exact integers and, the u_b being centred, of the result's
+// own size.
+template <int W>
+__device__ __forceinline__ void fold_voxel(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
+                                           uint64_t v, const FoldConst &fc, double &dv, double &sv,
+                                           unsigned long long &tot_out) {
+    unsigned long long s[W];
+    unsigned long long tot = 0;
 #pragma unroll
     for (int b = 0; b < W; ++b) {
         s[b] = __ldcs(tally + (uint64_t)b * nvox + v);
         tot += s[b];
-        add_sq(sq, s[b]);
     }
-    double var_sum;  // sum_b (S_b - S/W)^2, in quanta^2
-    if (sq.hi < (1ull << 57)) {
-        // W sum S_b^2 - S^2, exact and non-negative (Cauchy-Schwarz), = W var_sum
-        const U128 ws{sq.lo * (unsigned long long)W, sq.hi * (unsigned long long)W + __umul64hi(sq.lo, (unsigned long long)W)};
-        const U128 t2{tot * tot, __umul64hi(tot, tot)};
-        const U128 num{ws.lo - t2.lo, ws.hi - t2.hi - (ws.lo < t2.lo ? 1ull : 0ull)};
-        var_sum = u128_to_double(num) * (1.0 / (double)W);
-    } else {
-        const double m = (double)tot * (1.0 / (double)W);
-        double acc = 0.0;
-        for (int b = 0; b < W; ++b) {
-            const double t = (double)s[b] - m;
-            acc = fma(t, t, acc);
-        }
-        var_sum = acc;
-    }
-    // var(D) = var_sum / (W (W - 1) n^2) in quanta^2 per history^2
-    const double r = fc.k_dose / (double)(vox[v] >> 4);
-    dv = (double)tot * fc.inv_n * r;
-    sv = sqrt(var_sum * ((double)W * fc.c_var)) * r;
+    const uint32_t code = vox[v] >> 4;
     tot_out = tot;
+    dv = sv = 0.0;
+    if (tot == 0ull) return;
+    const double td = u128_to_double(U128{tot, 0ull});
+    const double a0 = td * fc.q_n;
+    const unsigned long long i = __double2ull_rn(a0);
+    U128 sq{0ull, 0ull};
+    long long u1 = 0;  // sum over the first r batches
+#pragma unroll
+    for (int b = 0; b < W; ++b) {
+        const long long u = (long long)(s[b] - i);
+        u1 += b < (int)fc.r ? u : 0ll;
+        add_sq(sq, (unsigned long long)(u < 0 ? -u : u));
+    }
+    double acc;
+    if (sq.hi < (1ull << 57)) {
+        const long long u0 = (long long)(tot - (unsigned long long)W * i) - u1;
+        const double f0 = a0 - __ull2double_rn(i), f1 = fma(td, fc.inv_n, f0);
+        const double r = (double)fc.r, w = (double)W - r;
+        acc = u128_to_double(sq);
+        acc = fma(f1, fma(r, f1, -2.0 * (double)u1), acc);
+        acc = fma(f0, fma(w, f0, -2.0 * (double)u0), acc);
+    } else {
+        acc = two_pass(tally, nvox, W, v, td, fc);
+    }
+    const double y = rcp_code(code);
+    dv = td * fc.k_dose * y;
+    sv = sqrt_fold(acc) * fc.k_sigma * y;
 }
 
-template <int W>
-__global__ void k_fold_equal(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox, FoldConst fc,
-                             double *dose, double *sigma, unsigned long long *dmax_bits,
-                             unsigned long long *dep_sum) {
-    double local_max = 0.0;
-    unsigned long long local_sum = 0;
+// CTAs of 256 threads an SM holds at the registers of each form (the sums of a
+// voxel live in registers with unequal batches); the grid is one full wave of
+// them, as a second partial one would cost as much as the first.
+template <int W, bool EQUAL>
+constexpr int kFoldBlocks = EQUAL ? 6 : W <= 16 ? 4 : W == 32 ? 2 : 1;
+
+template <int W, bool EQUAL>
+__global__ void __launch_bounds__(256, kFoldBlocks<W, EQUAL>) k_fold(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
+                                              FoldConst fc, double *dose, double *sigma,
+                                              unsigned long long *dmax_bits, unsigned long long *dep_sum) {
+    unsigned long long local_max = 0, local_sum = 0;  // doses are >= 0: their bits order as they do
     for (uint64_t v = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; v < nvox;
          v += (uint64_t)gridDim.x * blockDim.x) {
         double dv, sv;
         unsigned long long tot;
-        fold_voxel_equal<W>(tally, vox, nvox, v, fc, dv, sv, tot);
+        if (EQUAL)
+            fold_voxel_equal<W>(tally, vox, nvox, v, fc, dv, sv, tot);
+        else
+            fold_voxel<W>(tally, vox, nvox, v, fc, dv, sv, tot);
         if (dose) dose[v] = dv;
         if (sigma) sigma[v] = sv;
-        local_max = fmax(local_max, dv);
+        local_max = max(local_max, (unsigned long long)__double_as_longlong(dv));
         local_sum += tot;
     }
     for (int o = 16; o > 0; o >>= 1) {
-        local_max = fmax(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));
+        local_max = max(local_max, __shfl_xor_sync(0xffffffffu, local_max, o));
         local_sum += __shfl_xor_sync(0xffffffffu, local_sum, o);
     }
     if ((threadIdx.x & 31) == 0) {
-        atomicMax(dmax_bits, (unsigned long long)__double_as_longlong(local_max));
+        atomicMax(dmax_bits, local_max);
         if (local_sum) atomicAdd(dep_sum, local_sum);
     }
 }
@@ -621,50 +687,41 @@ cudaError_t launch_spectrum(const double *edges, const double *w, int n, float *
     return cudaGetLastError();
 }
 
-// Host side of both folds: the per-batch history counts and whether they are
-// all equal (the integer-variance form), and the constants of that form.
-static bool fold_args(int W, const double *n_b, FoldArgs &fa) {
-    bool equal = true;
-    for (int b = 0; b < 64; ++b) {
-        fa.n_b[b] = b < W ? n_b[b] : 0.0;
-        if (b < W && n_b[b] != n_b[0]) equal = false;
-    }
-    return equal;
-}
-
-static FoldConst fold_const(int W, double n_tot, double inv_vol) {
+// The fold's constants for N histories in W batches, each rounded once.
+static FoldConst fold_const(int W, uint64_t n_hist, double inv_vol) {
     FoldConst fc;
-    const double n = n_tot / (double)W;
-    fc.inv_n = 1.0 / n_tot;
-    fc.c_var = 1.0 / ((double)W * (double)W * (double)(W - 1) * n * n);
-    fc.k_dose = kQ * kMeVPerGramToGy * inv_vol / kRhoQ;
+    const long double N = (long double)n_hist;
+    fc.r = (uint32_t)(n_hist % (uint64_t)W);
+    fc.inv_n = (double)(1.0L / N);
+    fc.q_n = (double)((long double)(n_hist / (uint64_t)W) / N);
+    const long double k = (long double)kQ * kMeVPerGramToGy * inv_vol * (1.0L / (long double)kRhoQ) / N;
+    fc.k_dose = (double)k;
+    fc.k_sigma = (double)(k * sqrtl((fc.r ? (long double)W : 1.0L) / (long double)(W - 1)));
     return fc;
 }
 
-cudaError_t launch_fold(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox, int W,
-                        const double *n_b, double n_tot, double inv_vol, double *dose, double *sigma,
-                        unsigned long long *dmax_bits, unsigned long long *dep_sum, int n_sm, cudaStream_t s) {
-    FoldArgs fa;
-    const bool equal = fold_args(W, n_b, fa);
-    uint64_t blocks = (nvox + 255) / 256;
-    const uint64_t cap = (uint64_t)n_sm * 8;
-    const int grid = (int)(blocks < cap ? (blocks ? blocks : 1) : cap);
-    if (equal) {
-        const FoldConst fc = fold_const(W, n_tot, inv_vol);
-        switch (W) {
-            case 8: k_fold_equal<8><<<grid, 256, 0, s>>>(tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum); break;
-            case 16: k_fold_equal<16><<<grid, 256, 0, s>>>(tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum); break;
-            case 32: k_fold_equal<32><<<grid, 256, 0, s>>>(tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum); break;
-            case 64: k_fold_equal<64><<<grid, 256, 0, s>>>(tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum); break;
-            default: return cudaErrorInvalidValue;
-        }
-        return cudaGetLastError();
-    }
+template <int W>
+static void launch_fold_w(int n_sm, const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
+                          const FoldConst &fc, double *dose, double *sigma, unsigned long long *dmax_bits,
+                          unsigned long long *dep_sum, cudaStream_t s) {
+    const uint64_t blocks = nvox ? (nvox + 255) / 256 : 1;
+    const uint64_t wave = (uint64_t)n_sm * (fc.r == 0 ? kFoldBlocks<W, true> : kFoldBlocks<W, false>);
+    const int grid = (int)(blocks < wave ? blocks : wave);
+    if (fc.r == 0)
+        k_fold<W, true><<<grid, 256, 0, s>>>(tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum);
+    else
+        k_fold<W, false><<<grid, 256, 0, s>>>(tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum);
+}
+
+cudaError_t launch_fold(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox, int W, uint64_t n_hist,
+                        double inv_vol, double *dose, double *sigma, unsigned long long *dmax_bits,
+                        unsigned long long *dep_sum, int n_sm, cudaStream_t s) {
+    const FoldConst fc = fold_const(W, n_hist, inv_vol);
     switch (W) {
-        case 8: k_fold<8><<<grid, 256, 0, s>>>(tally, vox, nvox, fa, n_tot, inv_vol, dose, sigma, dmax_bits, dep_sum); break;
-        case 16: k_fold<16><<<grid, 256, 0, s>>>(tally, vox, nvox, fa, n_tot, inv_vol, dose, sigma, dmax_bits, dep_sum); break;
-        case 32: k_fold<32><<<grid, 256, 0, s>>>(tally, vox, nvox, fa, n_tot, inv_vol, dose, sigma, dmax_bits, dep_sum); break;
-        case 64: k_fold<64><<<grid, 128, 0, s>>>(tally, vox, nvox, fa, n_tot, inv_vol, dose, sigma, dmax_bits, dep_sum); break;
+        case 8: launch_fold_w<8>(n_sm, tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum, s); break;
+        case 16: launch_fold_w<16>(n_sm, tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum, s); break;
+        case 32: launch_fold_w<32>(n_sm, tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum, s); break;
+        case 64: launch_fold_w<64>(n_sm, tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum, s); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -707,8 +764,7 @@ cudaError_t launch_philox(const uint32_t *ctr, uint2 key, uint64_t n, int curand
 // ---------------------------------------------------------------------------
 // Allocation-free fold (gpumcd_plan_result_noalloc).
 //
-// The same dose / uncertainty fold as k_fold and k_fold_equal (the same
-// per-voxel functions), with its reduction scratch in a
+// The same dose / uncertainty fold as k_fold (the same per-voxel functions), with its reduction scratch in a
 // file-scope device array instead of device memory allocated at run time.
 // Each block folds one fixed range of voxels and writes its partial results
 // to its own slots of the array; single-block kernels then combine the
@@ -728,14 +784,12 @@ static_assert((uint64_t)kMaxBlocks * kVoxPerBlock == GPUMCD_NOALLOC_MAX_VOXELS, 
 // count) followed by 4 result words (D_max bits, deposited, s_thr bits, count).
 static __device__ __align__(256) unsigned long long scratch[kMaxBlocks * 4 + 4];
 
-// EQUAL selects the integer-variance form of k_fold_equal, else the form of
-// k_fold: the per-voxel arithmetic is the same function as the regular
-// fold's, so dose and sigma match gpumcd_plan_result's bit for bit.
+// The per-voxel arithmetic is the same function as the regular fold's, so
+// dose and sigma match gpumcd_plan_result's bit for bit.
 template <int W, bool EQUAL>
 __global__ void __launch_bounds__(kThreads) k_fold_blocks(const unsigned long long *tally, const uint32_t *vox,
-                                                          uint64_t nvox, const __grid_constant__ FoldArgs fa,
-                                                          FoldConst fc, double n_tot, double inv_vol, double *dose,
-                                                          double *sigma, unsigned long long *part) {
+                                                          uint64_t nvox, FoldConst fc, double *dose, double *sigma,
+                                                          unsigned long long *part) {
     __shared__ double smax[kThreads / 32];
     __shared__ unsigned long long ssum[kThreads / 32];
     const uint64_t v0 = blockIdx.x * kVoxPerBlock;
@@ -749,7 +803,7 @@ __global__ void __launch_bounds__(kThreads) k_fold_blocks(const unsigned long lo
         if (EQUAL)
             fold_voxel_equal<W>(tally, vox, nvox, v, fc, dv, sv, tot);
         else
-            fold_voxel<W>(tally, vox, nvox, v, fa, n_tot, inv_vol, dv, sv, tot);
+            fold_voxel<W>(tally, vox, nvox, v, fc, dv, sv, tot);
         dose[v] = dv;
         sigma[v] = sv;
         local_max = fmax(local_max, dv);
@@ -899,32 +953,30 @@ static unsigned long long *noalloc_scratch(int device, cudaError_t *err) {
 }
 
 template <int W>
-static void launch_fold_blocks(bool equal, int nb, cudaStream_t s, const unsigned long long *tally,
-                               const uint32_t *vox, uint64_t nvox, const FoldArgs &fa, const FoldConst &fc,
-                               double n_tot, double inv_vol, double *dose, double *sigma, unsigned long long *part) {
+static void launch_fold_blocks(int nb, cudaStream_t s, const unsigned long long *tally, const uint32_t *vox,
+                               uint64_t nvox, const FoldConst &fc, double *dose, double *sigma,
+                               unsigned long long *part) {
     using namespace noalloc;
-    if (equal)
-        k_fold_blocks<W, true><<<nb, kThreads, 0, s>>>(tally, vox, nvox, fa, fc, n_tot, inv_vol, dose, sigma, part);
+    if (fc.r == 0)
+        k_fold_blocks<W, true><<<nb, kThreads, 0, s>>>(tally, vox, nvox, fc, dose, sigma, part);
     else
-        k_fold_blocks<W, false><<<nb, kThreads, 0, s>>>(tally, vox, nvox, fa, fc, n_tot, inv_vol, dose, sigma, part);
+        k_fold_blocks<W, false><<<nb, kThreads, 0, s>>>(tally, vox, nvox, fc, dose, sigma, part);
 }
 
 cudaError_t launch_fold_noalloc(int device, const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
-                                int W, const double *n_b, double n_tot, double inv_vol, double thr, double *dose,
-                                double *sigma, cudaStream_t s, unsigned long long result[4]) {
+                                int W, uint64_t n_hist, double inv_vol, double thr, double *dose, double *sigma,
+                                cudaStream_t s, unsigned long long result[4]) {
     cudaError_t e = cudaSuccess;
     unsigned long long *part = noalloc_scratch(device, &e);
     if (!part) return e != cudaSuccess ? e : cudaErrorInvalidDevicePointer;
-    FoldArgs fa;
-    const bool equal = fold_args(W, n_b, fa);
-    const FoldConst fc = fold_const(W, n_tot, inv_vol);
+    const FoldConst fc = fold_const(W, n_hist, inv_vol);
     const int nb = (int)((nvox + noalloc::kVoxPerBlock - 1) / noalloc::kVoxPerBlock);
     using namespace noalloc;
     switch (W) {
-        case 8: launch_fold_blocks<8>(equal, nb, s, tally, vox, nvox, fa, fc, n_tot, inv_vol, dose, sigma, part); break;
-        case 16: launch_fold_blocks<16>(equal, nb, s, tally, vox, nvox, fa, fc, n_tot, inv_vol, dose, sigma, part); break;
-        case 32: launch_fold_blocks<32>(equal, nb, s, tally, vox, nvox, fa, fc, n_tot, inv_vol, dose, sigma, part); break;
-        case 64: launch_fold_blocks<64>(equal, nb, s, tally, vox, nvox, fa, fc, n_tot, inv_vol, dose, sigma, part); break;
+        case 8: launch_fold_blocks<8>(nb, s, tally, vox, nvox, fc, dose, sigma, part); break;
+        case 16: launch_fold_blocks<16>(nb, s, tally, vox, nvox, fc, dose, sigma, part); break;
+        case 32: launch_fold_blocks<32>(nb, s, tally, vox, nvox, fc, dose, sigma, part); break;
+        case 64: launch_fold_blocks<64>(nb, s, tally, vox, nvox, fc, dose, sigma, part); break;
         default: return cudaErrorInvalidValue;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
