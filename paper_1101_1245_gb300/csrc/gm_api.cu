@@ -91,6 +91,8 @@ struct Slot {
 
 }  // namespace
 
+constexpr int kRedWords = 16;  // the result block of a fold (launch_sthr)
+
 struct gpumcd_ctx {
     int device = 0;
     int n_sm = 0;
@@ -113,6 +115,7 @@ struct gpumcd_ctx {
     cudaEvent_t order = nullptr;  // orders a submitted sequence after the context stream
     int32_t next_ticket = 1;
     DevBuf fold_tmp;
+    unsigned long long *h_red = nullptr;  // pinned: the result block of the last fold
     std::multimap<size_t, void *> cache;  // freed device blocks by size
     uint64_t cached = 0;
     bool configured = false;
@@ -339,6 +342,7 @@ gpumcd_status gpumcd_init(gpumcd_ctx **out, int32_t device, uint64_t hbm_budget_
     if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&c->stream, cudaStreamNonBlocking, greatest);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->order, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaMallocHost(&c->h_red, kRedWords * sizeof(unsigned long long));
     if (e != cudaSuccess) {
         delete c;
         return cuda_status(e);
@@ -377,6 +381,7 @@ gpumcd_status gpumcd_destroy(gpumcd_ctx *c) {
     for (Slot &sl : c->slot) free_slot(c, sl);
     dev_free(c, c->fold_tmp);
     cache_trim(c, 0);
+    if (c->h_red) cudaFreeHost(c->h_red);
     if (c->order) cudaEventDestroy(c->order);
     if (c->stream) cudaStreamDestroy(c->stream);
     delete c;
@@ -1102,30 +1107,30 @@ gpumcd_status gpumcd_plan_result(gpumcd_ctx *c, int32_t plan_id, double thr, dou
     Plan &p = it->second;
     const Phantom &ph = c->phantoms.at(p.phantom);
     const uint64_t nvox = ph.nvox;
-    // scratch: [dose | sigma] when the caller passes NULL, then [dmax | sum | count | esum],
-    // then the s_thr reduction's per-block partials
-    const size_t need = (size_t)nvox * 16 + 64 + (size_t)sthr_blocks(nvox, c->n_sm) * 16;
+    // scratch: [dose | sigma] when the caller passes NULL, then the result
+    // block, then the s_thr reduction's per-block partials
+    const size_t need = (size_t)nvox * 16 + kRedWords * 8 + (size_t)sthr_blocks(nvox, c->n_sm) * 16;
     ST(dev_alloc(c, c->fold_tmp, need));
     double *tdose = (double *)c->fold_tmp.p;
     double *tsig = tdose + nvox;
     unsigned long long *red = (unsigned long long *)(tsig + nvox);
-    void *sthr_part = red + 8;
+    void *sthr_part = red + kRedWords;
     double *ddose = dose ? dose : tdose;
     double *dsig = sigma ? sigma : tsig;
     const uint64_t N = p.hist_done;
-    CK(cudaMemsetAsync(red, 0, 64, s));
+    CK(cudaMemsetAsync(red, 0, kRedWords * 8, s));
     const double inv_vol = 1.0 / (ph.voxel[0] * ph.voxel[1] * ph.voxel[2]);
     if (N > 0) {
         CK(launch_fold((const unsigned long long *)p.tally.p, (const uint32_t *)ph.vox.p, nvox, (int)p.W, N, inv_vol,
                        ddose, dsig, red, red + 3, c->n_sm, s));
-        CK(launch_sthr(ddose, dsig, nvox, red, thr, (double *)(red + 1), red + 2, sthr_part, c->n_sm, s));
+        CK(launch_sthr(ddose, dsig, nvox, thr, sthr_part, red, (const unsigned long long *)p.ledger.p, c->n_sm, s));
     } else {
         CK(cudaMemsetAsync(ddose, 0, nvox * 8, s));
         CK(cudaMemsetAsync(dsig, 0, nvox * 8, s));
+        CK(cudaMemcpyAsync(red + 5, p.ledger.p, 4 * 8, cudaMemcpyDeviceToDevice, s));
     }
-    unsigned long long h_red[4], h_led[4];
-    CK(cudaMemcpyAsync(h_red, red, sizeof h_red, cudaMemcpyDeviceToHost, s));
-    CK(cudaMemcpyAsync(h_led, p.ledger.p, sizeof h_led, cudaMemcpyDeviceToHost, s));
+    const unsigned long long *h_red = c->h_red, *h_led = c->h_red + 5;
+    CK(cudaMemcpyAsync(c->h_red, red, 9 * 8, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (stats) {
         *stats = p.acc;

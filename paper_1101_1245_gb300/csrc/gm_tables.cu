@@ -326,21 +326,22 @@ __global__ void k_spectrum(const double *edges, const double *w, int n, float *o
 //
 // GB300 issues two FP64 operations a clock and SM, so a voxel's FP64 work, not
 // its W x 8 bytes, bounded this kernel: about 31 operations a voxel (a
-// division, a square root and conversions among them) held it at 34% of the
-// copy rate.  Now the sums are formed in integers, rounded to FP64 by integer
-// instructions, and the division and square root start from the FP32
-// reciprocal and reciprocal square root and take one third-order step: 12
-// operations a voxel (about 25 with unequal batches, 85 before), none for a
-// voxel without dose, and dose and sigma are as close to the exact values as
-// before or closer.  A result call (fold, s_thr, read-back of the stats) of
-// 256^3 voxels, equal / unequal batches: 16 batches 0.53 / 0.97 ms (1.07 /
-// 3.00 before; the bytes alone take 0.37 at the copy rate), 64 batches 1.49 /
-// 2.36 ms (2.29 / 7.36; 1.32).
+// division, a square root and conversions among them; 85 with unequal batches)
+// held it at 34% of the copy rate.  Now the sums are formed in integers and
+// rounded to FP64 by integer instructions, the reciprocal of the density code
+// is integer work too, and the square root is one third-order step from the
+// FP32 reciprocal square root: 9 operations a voxel (13 with unequal batches),
+// none for a voxel without dose.  Dose and sigma are as close to the exact
+// values as before or closer.  A result call (fold, s_thr, read-back of the
+// stats) of 256^3 voxels, equal / unequal batches: 16 batches 0.48 / 0.62 ms
+// (1.07 / 3.00 before; the bytes alone take 0.37 at the copy rate), 64 batches
+// 1.41 / 1.45 ms (2.29 / 7.36; 1.32).
 struct FoldConst {
     double k_dose;   // (q * (MeV/g -> Gy) / (voxel volume * density quantum)) / N
     double k_sigma;  // ... times sqrt(W / (W - 1)) (unequal batches) or sqrt(1 / (W - 1)) (equal)
     double inv_n;    // 1 / N
     double q_n;      // (N div W) / N
+    double n1, n0;   // r and W - r
     uint32_t r;      // N mod W: the batches with one history more
 };
 
@@ -353,6 +354,29 @@ __device__ __forceinline__ void add_sq(U128 &acc, unsigned long long x) {
     const unsigned long long nl = acc.lo + lo;
     acc.hi += hi + (nl < lo ? 1ull : 0ull);
     acc.lo = nl;
+}
+
+// The sum and the sum of squares of K batch sums.  Sums below 2^32 quanta (64
+// MeV), most voxels', take one 32 x 32 multiplication each instead of four.
+template <int K>
+__device__ __forceinline__ void add_sums(const unsigned long long (&s)[K], unsigned long long &tot, U128 &sq) {
+    unsigned high = 0u;
+#pragma unroll
+    for (int b = 0; b < K; ++b) {
+        tot += s[b];
+        high |= (unsigned)(s[b] >> 32);
+    }
+    if (high == 0u) {
+#pragma unroll
+        for (int b = 0; b < K; ++b) {
+            const unsigned long long p = (unsigned long long)(unsigned)s[b] * (unsigned)s[b];
+            sq.lo += p;
+            sq.hi += sq.lo < p ? 1ull : 0ull;
+        }
+    } else {
+#pragma unroll
+        for (int b = 0; b < K; ++b) add_sq(sq, s[b]);
+    }
 }
 
 // v rounded to the nearest double (ties to even), by integer instructions.
@@ -377,15 +401,25 @@ __device__ __forceinline__ double float_to_double(float x) {  // normal x > 0
     return __hiloint2double((int)((b >> 3) + 0x38000000u), (int)(b << 29));
 }
 
-// 1 / code for 1 <= code < 2^28: the FP32 reciprocal y has a relative error e
-// below 2^-22, and y (1 + e + e^2) one of e^3.
+// x 2^k, negated when neg, by integer instructions.
+__device__ __forceinline__ double scaled(unsigned long long x, int k, bool neg) {
+    if (x == 0ull) return 0.0;
+    const double d = u128_to_double(U128{x, 0ull});
+    return __hiloint2double((__double2hiint(d) + (k << 20)) | (neg ? (int)0x80000000u : 0), __double2loint(d));
+}
+
+// 1 / code for 1 <= code < 2^28, in integers.  code = d 2^(31-n) with d in
+// [1, 2) held in units of 2^-31 (m); y0, the FP32 reciprocal of d in units of
+// 2^-32, is off by e = 1 - d y0 (below 2^-21), and y0 (1 + e + e^2), in units
+// of 2^-62, by e^3 and a few units.
 __device__ __forceinline__ double rcp_code(uint32_t code) {
     const int n = __clz((int)code);
     const uint32_t m = code << n;
-    const double d = __hiloint2double((int)(((uint32_t)(1053 - n) << 20) + (m >> 11)), (int)(m << 21));
-    const double y = float_to_double(__fdividef(1.0f, (float)code));
-    const double e = fma(-d, y, 1.0);
-    return fma(y, fma(e, e, e), y);
+    const uint32_t y0 = __float2uint_rz(__fdividef(9223372036854775808.0f, (float)m));  // 2^63 / m, saturating
+    const long long e = (long long)(0x8000000000000000ull - (unsigned long long)m * y0);  // in units of 2^-63
+    const long long t = e + (__mul64hi(e, e) << 1);
+    const unsigned long long y = ((unsigned long long)y0 << 30) + (unsigned long long)__mul64hi(t, (long long)y0 << 31);
+    return scaled(y, n - 62 - 31, false);
 }
 
 // sqrt(v) for v = 0 or normal v > 0: v = m 4^k with m in [1, 4), y the FP32
@@ -424,7 +458,7 @@ template <int W>
 __device__ __forceinline__ void fold_voxel_equal(const unsigned long long *tally, const uint32_t *vox,
                                                  uint64_t nvox, uint64_t v, const FoldConst &fc, double &dv,
                                                  double &sv, unsigned long long &tot_out) {
-    constexpr int K = W < 16 ? W : 16;  // loads in flight
+    constexpr int K = 8;  // loads in flight
     unsigned long long tot = 0;
     U128 sq{0ull, 0ull};
 #pragma unroll
@@ -432,11 +466,7 @@ __device__ __forceinline__ void fold_voxel_equal(const unsigned long long *tally
         unsigned long long s[K];
 #pragma unroll
         for (int b = 0; b < K; ++b) s[b] = __ldcs(tally + (uint64_t)(b0 + b) * nvox + v);
-#pragma unroll
-        for (int b = 0; b < K; ++b) {
-            tot += s[b];
-            add_sq(sq, s[b]);
-        }
+        add_sums(s, tot, sq);
     }
     const uint32_t code = vox[v] >> 4;
     tot_out = tot;
@@ -456,46 +486,66 @@ __device__ __forceinline__ void fold_voxel_equal(const unsigned long long *tally
     sv = sqrt_fold(num) * fc.k_sigma * y;
 }
 
-// Any batch counts: with i the integer nearest (N div W) D and u_b = S_b - i,
-// S_b - n_b D = u_b - f, where f = (N div W) D - i, plus D for the first r
-// batches; so
-//   sum_b (S_b - n_b D)^2 = sum u_b^2 + f1 (r f1 - 2 sum_{b<r} u_b) + f0 ((W-r) f0 - 2 sum_{b>=r} u_b),
-// whose sums are exact integers and, the u_b being centred, of the result's
-// own size.
+// Unequal batches: with i the integer nearest a0 = (N div W) D, f0 = a0 - i and
+// u_b = S_b - i, S_b - n_b D = u_b - f, where f is f0, plus D for the first r
+// batches; so, with U1 and U0 the sums of u_b over these and over the others,
+//   sum_b (S_b - n_b D)^2 = sum u_b^2 + f1 (r f1 - 2 U1) + f0 ((W-r) f0 - 2 U0).
+// The sums of u_b follow exactly, in 128-bit integers, from those of S_b, and,
+// the u_b being centred, the terms are of the result's own size.
 template <int W>
 __device__ __forceinline__ void fold_voxel(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
                                            uint64_t v, const FoldConst &fc, double &dv, double &sv,
                                            unsigned long long &tot_out) {
-    unsigned long long s[W];
-    unsigned long long tot = 0;
+    constexpr int K = 8;  // loads in flight
+    unsigned long long tot = 0, first = 0;  // sums over all and over the first r batches
+    U128 sq{0ull, 0ull};
 #pragma unroll
-    for (int b = 0; b < W; ++b) {
-        s[b] = __ldcs(tally + (uint64_t)b * nvox + v);
-        tot += s[b];
+    for (int b0 = 0; b0 < W; b0 += K) {
+        unsigned long long s[K];
+#pragma unroll
+        for (int b = 0; b < K; ++b) s[b] = __ldcs(tally + (uint64_t)(b0 + b) * nvox + v);
+        add_sums(s, tot, sq);
+#pragma unroll
+        for (int b = 0; b < K; ++b) first += b0 + b < (int)fc.r ? s[b] : 0ull;
     }
     const uint32_t code = vox[v] >> 4;
     tot_out = tot;
     dv = sv = 0.0;
     if (tot == 0ull) return;
     const double td = u128_to_double(U128{tot, 0ull});
-    const double a0 = td * fc.q_n;
-    const unsigned long long i = __double2ull_rn(a0);
-    U128 sq{0ull, 0ull};
-    long long u1 = 0;  // sum over the first r batches
-#pragma unroll
-    for (int b = 0; b < W; ++b) {
-        const long long u = (long long)(s[b] - i);
-        u1 += b < (int)fc.r ? u : 0ll;
-        add_sq(sq, (unsigned long long)(u < 0 ? -u : u));
-    }
     double acc;
     if (sq.hi < (1ull << 57)) {
-        const long long u0 = (long long)(tot - (unsigned long long)W * i) - u1;
-        const double f0 = a0 - __ull2double_rn(i), f1 = fma(td, fc.inv_n, f0);
-        const double r = (double)fc.r, w = (double)W - r;
-        acc = u128_to_double(sq);
-        acc = fma(f1, fma(r, f1, -2.0 * (double)u1), acc);
-        acc = fma(f0, fma(w, f0, -2.0 * (double)u0), acc);
+        const double a0 = td * fc.q_n;
+        // i and f0 from a0's bits (its exponent is below 63: a0 < S / W)
+        const int ex = (__double2hiint(a0) >> 20) - 1023;
+        const unsigned long long m = ((unsigned long long)__double_as_longlong(a0) << 11) | (1ull << 63);  // a0 = m 2^(ex-63)
+        unsigned long long i = 0ull;
+        double f0 = a0;
+        if (ex >= -1) {
+            i = ex >= 0 ? m >> (63 - ex) : 0ull;
+            unsigned long long f = ex >= 0 ? m << 1 << ex : m;  // the bits below, in units of 2^-64
+            const bool up = (f >> 63) != 0ull;
+            if (up) {
+                ++i;
+                f = 0ull - f;
+            }
+            f0 = scaled(f, -64, up);
+        }
+        // sum u_b^2 = sum S_b^2 - i (2 S - W i)
+        const unsigned long long wi = (unsigned long long)W * i;
+        const unsigned long long p1_lo = i * tot, p1_hi = __umul64hi(i, tot), p2_lo = i * wi, p2_hi = __umul64hi(i, wi);
+        U128 q = sq;
+        const unsigned long long d_lo = p1_lo << 1, d_hi = (p1_hi << 1) | (p1_lo >> 63);
+        q.hi -= d_hi + (q.lo < d_lo ? 1ull : 0ull);
+        q.lo -= d_lo;
+        q.lo += p2_lo;
+        q.hi += p2_hi + (q.lo < p2_lo ? 1ull : 0ull);
+        const long long u1 = (long long)(first - (unsigned long long)fc.r * i);
+        const long long u0 = (long long)(tot - wi) - u1;
+        const double f1 = fma(td, fc.inv_n, f0);
+        acc = u128_to_double(q);
+        acc = fma(f1, fma(fc.n1, f1, scaled((unsigned long long)(u1 < 0 ? -u1 : u1), 1, u1 > 0)), acc);
+        acc = fma(f0, fma(fc.n0, f0, scaled((unsigned long long)(u0 < 0 ? -u0 : u0), 1, u0 > 0)), acc);
     } else {
         acc = two_pass(tally, nvox, W, v, td, fc);
     }
@@ -504,14 +554,12 @@ __device__ __forceinline__ void fold_voxel(const unsigned long long *tally, cons
     sv = sqrt_fold(acc) * fc.k_sigma * y;
 }
 
-// CTAs of 256 threads an SM holds at the registers of each form (the sums of a
-// voxel live in registers with unequal batches); the grid is one full wave of
+// CTAs of 256 threads an SM holds (48 registers); the grid is one full wave of
 // them, as a second partial one would cost as much as the first.
-template <int W, bool EQUAL>
-constexpr int kFoldBlocks = EQUAL ? 6 : W <= 16 ? 4 : W == 32 ? 2 : 1;
+constexpr int kFoldBlocks = 5;
 
 template <int W, bool EQUAL>
-__global__ void __launch_bounds__(256, kFoldBlocks<W, EQUAL>) k_fold(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
+__global__ void __launch_bounds__(256, kFoldBlocks) k_fold(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
                                               FoldConst fc, double *dose, double *sigma,
                                               unsigned long long *dmax_bits, unsigned long long *dep_sum) {
     unsigned long long local_max = 0, local_sum = 0;  // doses are >= 0: their bits order as they do
@@ -539,31 +587,37 @@ __global__ void __launch_bounds__(256, kFoldBlocks<W, EQUAL>) k_fold(const unsig
 }
 
 // s_thr = mean of sigma/D over voxels with D > thr * D_max (GPUMCD §II.D, s).
-// Each block writes its partial sum and count to its own slot; one block then
-// adds the slots in a fixed order, so s_thr is the same bit for bit for the
-// same tally (the run-to-uncertainty schedule depends on it).
+// Each block writes its partial sum and count to its own slot; the block that
+// finishes last adds the slots in a fixed order, so s_thr is the same bit for
+// bit for the same tally (the run-to-uncertainty schedule depends on it), and
+// completes the result block: [D_max bits | sum | count | deposited | blocks
+// done | the plan's ledger (4)], which the host reads in one copy.  Doses are
+// >= 0, so they are compared as integers: as doubles, the two comparisons a
+// voxel kept the FP64 pipe busy for 85 us at 256^3, where the doses take 20 us
+// to read.
 constexpr int kSthrThreads = 256;
 
 __global__ void __launch_bounds__(kSthrThreads) k_sthr(const double *dose, const double *sigma, uint64_t nvox,
-                                                       const unsigned long long *dmax_bits, double thr,
-                                                       double2 *part) {
-    __shared__ double ss[kSthrThreads / 32];
-    __shared__ double sc[kSthrThreads / 32];
-    const double cut = thr * __longlong_as_double((long long)*dmax_bits);
+                                                       double thr, double2 *part, unsigned long long *red,
+                                                       const unsigned long long *ledger) {
+    __shared__ double ss[kSthrThreads];
+    __shared__ double sc[kSthrThreads];
+    __shared__ int last;
+    const double cut = thr * __longlong_as_double((long long)red[0]);
+    const unsigned long long cut_bits = (unsigned long long)__double_as_longlong(cut) & ~(1ull << 63);
+    const unsigned long long *bits = (const unsigned long long *)dose;
     double s = 0.0;
-    unsigned long long c = 0;
+    unsigned c = 0;
     for (uint64_t v = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; v < nvox;
          v += (uint64_t)gridDim.x * blockDim.x) {
-        const double d = dose[v];
-        if (d > cut && d > 0.0) {
-            s += sigma[v] / d;
+        const unsigned long long d = bits[v];
+        if (d > cut_bits) {
+            s += sigma[v] / __longlong_as_double((long long)d);
             ++c;
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        s += __shfl_xor_sync(0xffffffffu, s, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    c = __reduce_add_sync(0xffffffffu, c);
     if ((threadIdx.x & 31) == 0) {
         ss[threadIdx.x >> 5] = s;
         sc[threadIdx.x >> 5] = (double)c;
@@ -576,17 +630,17 @@ __global__ void __launch_bounds__(kSthrThreads) k_sthr(const double *dose, const
             b += sc[i];
         }
         part[blockIdx.x] = make_double2(a, b);
+        __threadfence();
+        last = atomicAdd(&red[4], 1ull) == gridDim.x - 1ull;
     }
-}
-
-__global__ void __launch_bounds__(kSthrThreads) k_sthr_combine(const double2 *part, int n, double *sum,
-                                                               unsigned long long *count) {
-    __shared__ double ss[kSthrThreads];
-    __shared__ double sc[kSthrThreads];
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
     double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < n; i += kSthrThreads) {
-        a += part[i].x;
-        b += part[i].y;
+    for (unsigned i = threadIdx.x; i < gridDim.x; i += kSthrThreads) {
+        const double2 p = __ldcg(part + i);
+        a += p.x;
+        b += p.y;
     }
     ss[threadIdx.x] = a;
     sc[threadIdx.x] = b;
@@ -599,9 +653,10 @@ __global__ void __launch_bounds__(kSthrThreads) k_sthr_combine(const double2 *pa
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        *sum = ss[0];
-        *count = (unsigned long long)sc[0];
+        red[1] = (unsigned long long)__double_as_longlong(ss[0]);
+        red[2] = (unsigned long long)sc[0];
     }
+    if (threadIdx.x < 4) red[5 + threadIdx.x] = ledger[threadIdx.x];
 }
 
 // Exact integer sum of a tally (for the energy ledger).
@@ -692,6 +747,8 @@ static FoldConst fold_const(int W, uint64_t n_hist, double inv_vol) {
     FoldConst fc;
     const long double N = (long double)n_hist;
     fc.r = (uint32_t)(n_hist % (uint64_t)W);
+    fc.n1 = (double)fc.r;
+    fc.n0 = (double)(W - (int)fc.r);
     fc.inv_n = (double)(1.0L / N);
     fc.q_n = (double)((long double)(n_hist / (uint64_t)W) / N);
     const long double k = (long double)kQ * kMeVPerGramToGy * inv_vol * (1.0L / (long double)kRhoQ) / N;
@@ -705,7 +762,7 @@ static void launch_fold_w(int n_sm, const unsigned long long *tally, const uint3
                           const FoldConst &fc, double *dose, double *sigma, unsigned long long *dmax_bits,
                           unsigned long long *dep_sum, cudaStream_t s) {
     const uint64_t blocks = nvox ? (nvox + 255) / 256 : 1;
-    const uint64_t wave = (uint64_t)n_sm * (fc.r == 0 ? kFoldBlocks<W, true> : kFoldBlocks<W, false>);
+    const uint64_t wave = (uint64_t)n_sm * kFoldBlocks;
     const int grid = (int)(blocks < wave ? blocks : wave);
     if (fc.r == 0)
         k_fold<W, true><<<grid, 256, 0, s>>>(tally, vox, nvox, fc, dose, sigma, dmax_bits, dep_sum);
@@ -733,12 +790,9 @@ int sthr_blocks(uint64_t nvox, int n_sm) {
     return (int)(blocks < cap ? (blocks ? blocks : 1) : cap);
 }
 
-cudaError_t launch_sthr(const double *dose, const double *sigma, uint64_t nvox,
-                        const unsigned long long *dmax_bits, double thr, double *sum,
-                        unsigned long long *count, void *part, int n_sm, cudaStream_t s) {
-    const int grid = sthr_blocks(nvox, n_sm);
-    k_sthr<<<grid, kSthrThreads, 0, s>>>(dose, sigma, nvox, dmax_bits, thr, (double2 *)part);
-    k_sthr_combine<<<1, kSthrThreads, 0, s>>>((const double2 *)part, grid, sum, count);
+cudaError_t launch_sthr(const double *dose, const double *sigma, uint64_t nvox, double thr, void *part,
+                        unsigned long long *red, const unsigned long long *ledger, int n_sm, cudaStream_t s) {
+    k_sthr<<<sthr_blocks(nvox, n_sm), kSthrThreads, 0, s>>>(dose, sigma, nvox, thr, (double2 *)part, red, ledger);
     return cudaGetLastError();
 }
 
@@ -862,6 +916,7 @@ __global__ void k_sthr_blocks(const double *dose, const double *sigma, uint64_t 
     __shared__ double ss[kThreads / 32];
     __shared__ unsigned long long sc[kThreads / 32];
     const double cut = thr * __longlong_as_double((long long)part[4 * kMaxBlocks + 0]);
+    const unsigned long long cut_bits = (unsigned long long)__double_as_longlong(cut) & ~(1ull << 63);
     const uint64_t v0 = blockIdx.x * kVoxPerBlock;
     double s = 0.0;
     unsigned long long c = 0;
@@ -869,7 +924,7 @@ __global__ void k_sthr_blocks(const double *dose, const double *sigma, uint64_t 
         const uint64_t v = v0 + (uint64_t)k * kThreads + threadIdx.x;
         if (v >= nvox) break;
         const double d = dose[v];
-        if (d > cut && d > 0.0) {
+        if ((unsigned long long)__double_as_longlong(d) > cut_bits) {  // as in k_sthr
             s += sigma[v] / d;
             ++c;
         }
