@@ -888,6 +888,8 @@ gpumcd_status seq_start(gpumcd_ctx *c, Slot &sl, int32_t n_plans, const int32_t 
     A.phys = c->dphys;
     A.plans = (const PlanDev *)sl.plandev.p;
     A.n_plans = n_plans;
+    for (int r = 0; r < 10; ++r)
+        A.round_key[r] = philox_round_key(make_uint2(sl.h_plandev[0].key_lo, sl.h_plandev[0].key_hi), r);
     A.prim_cursor = dc->prim_cursor;
     A.stacks = (Rec *)sl.stacks.p;
     A.hard = (HardRec *)sl.hard.p;

@@ -140,6 +140,7 @@ struct TransportArgs {
     uint32_t flags;
     uint32_t refill_period;            // 1: refill every pass; N: every N-th pass or when empty
     uint32_t phsp;                     // a plan of the launch has a phase-space source
+    uint2 round_key[10];               // one plan in the launch: its Philox round keys
     uint32_t tab_bytes;                // bytes of tables staged into shared memory (the loaded materials')
     unsigned long long *counters;      // run counters (see CNT_*)
     int32_t *error;                    // device status word
@@ -163,9 +164,16 @@ enum {
 // Philox4x32-10 (Salmon et al., SC'11): 10 rounds of the two 32x32->64
 // multiplies with the Weyl-sequence key schedule.
 // ---------------------------------------------------------------------------
-__host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
+__host__ __device__ __forceinline__ uint2 philox_round_key(uint2 k, int r) {
+    return make_uint2(k.x + (uint32_t)r * 0x9E3779B9u, k.y + (uint32_t)r * 0xBB67AE85u);
+}
+
+// key(r) is the key of round r.
+template <class RoundKey>
+__host__ __device__ __forceinline__ uint4 philox4x32_10_keyed(uint4 c, const RoundKey &key) {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
+        const uint2 k = key(r);
 #ifdef __CUDA_ARCH__
         const uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
         const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
@@ -175,10 +183,12 @@ __host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
         const uint32_t hi1 = (uint32_t)(p1 >> 32), lo1 = (uint32_t)p1;
 #endif
         c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
-        k.x += 0x9E3779B9u;
-        k.y += 0xBB67AE85u;
     }
     return c;
+}
+
+__host__ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
+    return philox4x32_10_keyed(c, [k](int r) { return philox_round_key(k, r); });
 }
 
 // Uniform in (0, 1] from the top 24 bits of a word.

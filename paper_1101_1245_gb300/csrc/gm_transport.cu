@@ -84,9 +84,27 @@ __device__ __forceinline__ float interp_ms(const float *t, float x) {
     return fmaf(f, t[i + 1] - t[i], t[i]);
 }
 
-__device__ __forceinline__ uint4 draw4(Lane &p, const PlanDev &P) {
-    const uint4 r = philox4x32_10(make_uint4(p.draw, p.lin_lo, p.lin_hi, p.hist),
-                                  make_uint2(P.key_lo, P.key_hi));
+// A plan's Philox round keys: computed from the plan's key (18 additions a
+// draw), or, in a launch of one plan (ONE), operands of the rounds' exclusive
+// ors in the kernel's arguments.  A draw's ten rounds are about a quarter of
+// the transport's time (a build with six is 9-11% faster).  ONE takes 1e6 15
+// MeV electrons on 128^3 water from 1.77 to 1.74 ms, 4e6 photons from 4.10 to
+// 4.00 ms, 4e6 photons on the slabs from 3.12 to 3.05 ms, and needs no spills.
+// Only the keys are read there: with the plan's other fields in the arguments
+// too, the compiler contracts other multiply-adds (the tallies move) and the
+// beams above take 0.4% more to 1.8% less than without ONE.
+template <bool ONE>
+struct RoundKeys {
+    const TransportArgs &A;
+    const PlanDev &P;
+    __device__ __forceinline__ uint2 operator()(int r) const {
+        return ONE ? A.round_key[r] : philox_round_key(make_uint2(P.key_lo, P.key_hi), r);
+    }
+};
+
+template <class Keys>
+__device__ __forceinline__ uint4 draw4(Lane &p, const Keys &key) {
+    const uint4 r = philox4x32_10_keyed(make_uint4(p.draw, p.lin_lo, p.lin_hi, p.hist), key);
     ++p.draw;
     return r;
 }
@@ -265,7 +283,8 @@ __device__ __forceinline__ Rec make_rec(const Lane &p) {
 // fourth word of the last draw in *w4.
 constexpr int SAMPLER_CAP = 4096;  // proposals before a sampler gives up (counted, never expected)
 
-__device__ float sample_kn(Lane &p, const PlanDev &P, float k, float *c, uint32_t *w4, unsigned *capped) {
+template <class Keys>
+__device__ float sample_kn(Lane &p, const Keys &P, float k, float *c, uint32_t *w4, unsigned *capped) {
     const float e0 = __fdividef(1.0f, 1.0f + 2.0f * k);
     const float a1 = __logf(1.0f + 2.0f * k);
     const float a2 = 0.5f * (1.0f - e0 * e0);
@@ -290,7 +309,8 @@ __device__ float sample_kn(Lane &p, const PlanDev &P, float k, float *c, uint32_
 
 // Sauter photo-electron polar angle (§II.A): nu = 1 - cos drawn from
 // nu/(A+nu)^3 and accepted with (2-nu)(1/(A+nu)+B) / (2(1/A+B)).
-__device__ float sample_sauter(Lane &p, const PlanDev &P, float T, uint32_t *w3, unsigned *capped) {
+template <class Keys>
+__device__ float sample_sauter(Lane &p, const Keys &P, float T, uint32_t *w3, unsigned *capped) {
     const float g = 1.0f + T / kMC2f;
     const float b2 = 1.0f - __fdividef(1.0f, g * g);
     const float beta = sqrtf(b2);
@@ -316,7 +336,8 @@ __device__ float sample_sauter(Lane &p, const PlanDev &P, float T, uint32_t *w3,
 // (4/3 - 4y/3 + y^2) cA + (1 - y) cB.  One loop serves both, so the lanes of a
 // warp share each proposal's draw (ten Philox rounds, most of a proposal)
 // whichever kind they sample.
-__device__ __forceinline__ float sample_hard(Lane &p, const PlanDev &P, bool moller, float T, float thr, float cA,
+template <class Keys>
+__device__ __forceinline__ float sample_hard(Lane &p, const Keys &P, bool moller, float T, float thr, float cA,
                                              float cB, uint32_t *w3, unsigned *capped) {
     float v0, v1, v2, v3;  // Moller: thr / T, c1, c2, bound; bremsstrahlung: E, ln(T / thr), cA, cB
     if (moller) {
@@ -385,14 +406,14 @@ __device__ __forceinline__ float sample_spectrum(const PlanDev &P, float z) {
 // so the draw counter starts where the beams' does).  A source grouped by
 // energy starts each history as an ungrouped one does: the grouping orders the
 // claims (refill), not the sample.
-template <bool PHSP>
-__device__ __forceinline__ uint32_t make_primary(Lane &p, const PlanDev &P, uint32_t plan, uint64_t h) {
+template <bool PHSP, bool ONE>
+__device__ __forceinline__ uint32_t make_primary(const TransportArgs &A, Lane &p, const PlanDev &P, uint32_t plan, uint64_t h) {
     p.hist = (uint32_t)h;
     p.lin_lo = 1u;
     p.lin_hi = 0u;
     p.draw = 0u;
     p.plan = plan;
-    const uint4 r = draw4(p, P);
+    const uint4 r = draw4(p, RoundKeys<ONE>{A, P});
     if (PHSP && P.beam == GPUMCD_BEAM_PHASE_SPACE) {
         const float4 *ps = reinterpret_cast<const float4 *>(P.spec);
         const uint32_t k = (uint32_t)(h % (unsigned long long)P.n_phsp);
@@ -433,12 +454,13 @@ __device__ __forceinline__ uint32_t make_primary(Lane &p, const PlanDev &P, uint
 // once for all flights of a pass: the energy does not change on a fictitious
 // event.  photon_interact: that interaction (Compton, photoelectric or pair,
 // by the partial attenuation coefficients of the voxel's material).
+template <bool ONE>
 __device__ __forceinline__ bool photon_flight(const TransportArgs &A, const Smem &S, Lane &p, float xp,
                                               float mu_hat, uint32_t &idx_out, uint32_t &rz, int &m_out,
                                               float &rho_out, float &mu_out, int w) {
     const PlanDev &P = S.plans[p.plan];
     const Phys &ph = A.phys;
-    const uint4 r = draw4(p, P);
+    const uint4 r = draw4(p, RoundKeys<ONE>{A, P});
     const float s = __fdividef(-__logf(u01(r.x)), mu_hat);
     p.x = fmaf(s, p.ux, p.x);
     p.y = fmaf(s, p.uy, p.y);
@@ -467,7 +489,7 @@ __device__ __forceinline__ bool photon_flight(const TransportArgs &A, const Smem
     return true;
 }
 
-template <bool KERMA>
+template <bool KERMA, bool ONE>
 __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Smem &S, Lane &p, uint32_t idx,
                                                 uint32_t rz, float xp, int m, float rho, float mu, int gw,
                                                 int w) {
@@ -485,7 +507,7 @@ __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Sm
         float c;
         uint32_t w4;
         unsigned capped = 0;
-        const float eps = sample_kn(p, P, E / kMC2f, &c, &w4, &capped);
+        const float eps = sample_kn(p, RoundKeys<ONE>{A, P}, E / kMC2f, &c, &w4, &capped);
         if (capped) count(S, w, CNT_SAMPLER_CAP);
         float sp, cp;
         __sincosf(kTWO_PIf * u01(w4), &sp, &cp);
@@ -517,7 +539,7 @@ __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Sm
         if (p.E >= ph.e_abs_q) {
             uint32_t w3;
             unsigned capped = 0;
-            const float c = sample_sauter(p, P, E, &w3, &capped);
+            const float c = sample_sauter(p, RoundKeys<ONE>{A, P}, E, &w3, &capped);
             if (capped) count(S, w, CNT_SAMPLER_CAP);
             float sp, cp;
             __sincosf(kTWO_PIf * u01(w3), &sp, &cp);
@@ -535,7 +557,7 @@ __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Sm
         count(S, w, CNT_PAIR);
         const uint32_t tt = p.E - ph.two_mc2_q;
         ledger_add(S, p.plan, 2, ph.two_mc2_q);
-        const uint4 r2 = draw4(p, P);
+        const uint4 r2 = draw4(p, RoundKeys<ONE>{A, P});
         const uint32_t t1 = min(tt, __float2uint_rn(u01(r2.x) * (float)tt));
         const uint32_t t2 = tt - t1;
         float sp, cp;
@@ -569,6 +591,7 @@ __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Sm
 // particle.  It starts above the absorption energy (the caller tests it).  A
 // step that ends outside or below that energy sets fin and leaves the end
 // point and the energy in p, for electron_end.
+template <bool ONE>
 __device__ __forceinline__ void electron_step(const TransportArgs &A, const Smem &S, Lane &p, int gw, int w,
                                               uint32_t &dep_idx, uint32_t &dep_e, bool &fin) {
     const PlanDev &P = S.plans[p.plan];
@@ -577,7 +600,7 @@ __device__ __forceinline__ void electron_step(const TransportArgs &A, const Smem
     const uint32_t idx0 = voxel_index(P, p.x, p.y, p.z, ix, iy, iz);
     const uint32_t vw = __ldg(P.vox + idx0);
     // the step's draw, taken while the voxel word is on its way
-    const uint4 r = draw4(p, P);
+    const uint4 r = draw4(p, RoundKeys<ONE>{A, P});
     const int m0 = vw & (NMAT - 1);
     const float rho0 = (float)(vw >> 4) * kRhoQ;
     const float *te = S.tab + tab_el(m0);
@@ -661,6 +684,7 @@ __device__ __forceinline__ void electron_end(const Smem &S, const Lane &p) {
 // voxel, which holds the candidate point (the step ends inside it, or at most
 // the nudge past its face) and so the event and its sub-cut-off deposits.
 // ---------------------------------------------------------------------------
+template <bool ONE>
 __device__ __forceinline__ void hard_event(const TransportArgs &A, const Smem &S, Lane &p, float sig_hat,
                                         uint32_t idx1, int gw, int w) {
     const PlanDev &P = S.plans[p.plan];
@@ -668,7 +692,7 @@ __device__ __forceinline__ void hard_event(const TransportArgs &A, const Smem &S
     const uint32_t e1 = p.E;
     // electron Woodcock: accept a real hard event with Sigma(T_end)/Sigma_hat
     const uint32_t vw1 = __ldg(P.vox + idx1);
-    const uint4 r2 = draw4(p, P);  // the event's draw, taken while the voxel word loads
+    const uint4 r2 = draw4(p, RoundKeys<ONE>{A, P});  // the event's draw, taken while the voxel word loads
     const int m1 = vw1 & (NMAT - 1);
     const float rho1 = (float)(vw1 >> 4) * kRhoQ;
     const float *t1 = S.tab + tab_el(m1);
@@ -693,7 +717,7 @@ __device__ __forceinline__ void hard_event(const TransportArgs &A, const Smem &S
     // and 4.09.
     uint32_t w3;
     unsigned capped = 0;
-    const float x = sample_hard(p, P, moller, T1, moller ? ph.t_c : ph.k_c, S.tab[TAB_BREM + 2 * m1],
+    const float x = sample_hard(p, RoundKeys<ONE>{A, P}, moller, T1, moller ? ph.t_c : ph.k_c, S.tab[TAB_BREM + 2 * m1],
                                 S.tab[TAB_BREM + 2 * m1 + 1], &w3, &capped);
     if (capped) count(S, w, CNT_SAMPLER_CAP);
     uint32_t e2;
@@ -798,7 +822,7 @@ __device__ void spill_to_queue(const TransportArgs &A, const Smem &S, int gw, in
 
 // Fill empty lanes with particles of type t.  Returns the number of lanes
 // that hold a particle afterwards.
-template <bool KERMA, bool PHSP>
+template <bool KERMA, bool PHSP, bool ONE>
 __device__ int refill(const TransportArgs &A, const Smem &S, CtaFlags &F, Lane &p, int gw, int w, int t) {
     const int lane = threadIdx.x & 31;
     WarpState &ws = S.ws[w];
@@ -873,7 +897,7 @@ __device__ int refill(const TransportArgs &A, const Smem &S, CtaFlags &F, Lane &
             // a source grouped by energy: its histories are claimed in
             // decreasing order of their energy (the order its launch sorted)
             if (PHSP && P.e_group && j < P.n_sorted) j = __ldg(P.order + j);
-            ledger_add(S, plan, 0, make_primary<PHSP>(p, P, plan, P.hist_base + j));
+            ledger_add(S, plan, 0, make_primary<PHSP, ONE>(A, p, P, plan, P.hist_base + j));
             if (t == 0 && p.E < A.phys.p_cut_q) {
                 // a photon primary below the photon cut-off deposits where it
                 // starts, or escapes from outside (every other photon flies
@@ -942,6 +966,7 @@ __device__ __forceinline__ unsigned available(const TransportArgs &A, const Smem
 // to 32 parked hard-event candidates into the lanes and run their events
 // together.  The lanes then hold electrons again (after their events), so
 // the warp goes on stepping electrons.
+template <bool ONE>
 __device__ __forceinline__ void hard_pass(const TransportArgs &A, const Smem &S, Lane &p, int gw, int w) {
     const int lane = threadIdx.x & 31;
     if (S.ws[w].stk[1] + 32u > A.stack_cap) spill_to_queue(A, S, gw, w, 1, 64u);
@@ -973,7 +998,7 @@ __device__ __forceinline__ void hard_pass(const TransportArgs &A, const Smem &S,
     // headroom for the events' secondaries (at most one per lane per type)
     if (S.ws[w].stk[0] + 64u > A.stack_cap) spill_to_queue(A, S, gw, w, 0, 64u);
     if (S.ws[w].stk[1] + 64u > A.stack_cap) spill_to_queue(A, S, gw, w, 1, 64u);
-    if (p.act) hard_event(A, S, p, sig_hat, idx1, gw, w);
+    if (p.act) hard_event<ONE>(A, S, p, sig_hat, idx1, gw, w);
     __syncwarp();
 }
 
@@ -1002,9 +1027,10 @@ __device__ __forceinline__ uint32_t smem_addr(const void *p) {
 // PROF compiles in the per-type cycle profile (GPUMCD_LAUNCH_PROFILE), AGG
 // the warp-aggregated deposit (GPUMCD_LAUNCH_WARP_AGGREGATE), SCHED the
 // refill policies of the divergence-reduction ablation (refill_period != 1),
-// KERMA the photon-only mode (GPUMCD_LAUNCH_KERMA) and PHSP phase-space
-// sources; the production instantiations carry none of them.
-template <int MAXT, int MINB, bool PROF, bool AGG, bool SCHED, bool KERMA, bool PHSP>
+// KERMA the photon-only mode (GPUMCD_LAUNCH_KERMA), PHSP phase-space sources
+// and ONE launches of one plan; the production instantiations carry none of
+// the first five.
+template <int MAXT, int MINB, bool PROF, bool AGG, bool SCHED, bool KERMA, bool PHSP, bool ONE>
 __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant__ TransportArgs A) {
     // the fixed-size parts first, at offsets known at compile time; the tables
     // of the loaded materials after them
@@ -1099,10 +1125,10 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
                 n_act = __popc(actm);
                 fresh = false;
             } else {
-                n_act = refill<KERMA, PHSP>(A, S, F, p, gw, w, t);
+                n_act = refill<KERMA, PHSP, ONE>(A, S, F, p, gw, w, t);
             }
         } else {
-            n_act = refill<KERMA, PHSP>(A, S, F, p, gw, w, t);
+            n_act = refill<KERMA, PHSP, ONE>(A, S, F, p, gw, w, t);
         }
         if (prof && lane == 0) atomicAdd(&S.cnt[CNT_PROF_REFILL_CYC], (unsigned long long)(clock64() - c0));
         const int o = 1 - t;
@@ -1116,7 +1142,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
             // iteration; n_act == 0 keeps parked candidates from being left
             // behind (also when refill_low is 0).
             if (hc >= 32u || (hc > 0u && (n_act == 0 || (n_act < (int)A.refill_low && hc >= (unsigned)n_act)))) {
-                hard_pass(A, S, p, gw, w);
+                hard_pass<ONE>(A, S, p, gw, w);
                 continue;
             }
         }
@@ -1170,10 +1196,10 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
                 if (flym == 0u) break;
                 if (fly) {
                     count(S, w, CNT_PH_EVENTS);
-                    real = photon_flight(A, S, p, xp, mu_hat, pidx, prz, rm, rrho, rmu, w);
+                    real = photon_flight<ONE>(A, S, p, xp, mu_hat, pidx, prz, rm, rrho, rmu, w);
                 }
             }
-            if (real) photon_interact<KERMA>(A, S, p, pidx, prz, xp, rm, rrho, rmu, gw, w);
+            if (real) photon_interact<KERMA, ONE>(A, S, p, pidx, prz, xp, rm, rrho, rmu, gw, w);
         } else {
             // Up to EL_STEPS steps before the warp goes back to refill its
             // lanes, as long as three quarters of them are still stepping.
@@ -1185,7 +1211,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
                 uint32_t dep_idx = 0, dep_e = 0;
                 if (p.act) {
                     count(S, w, CNT_E_STEPS);
-                    electron_step(A, S, p, gw, w, dep_idx, dep_e, fin);
+                    electron_step<ONE>(A, S, p, gw, w, dep_idx, dep_e, fin);
                 }
                 const PlanDev &P = S.plans[p.plan];
                 if (agg)
@@ -1229,27 +1255,33 @@ size_t transport_smem_bytes(uint32_t tab_bytes) { return (size_t)SMEM_FIXED + ta
 // workload than 512 x 2 in a same-box A/B).  The profile, aggregation,
 // refill-policy, photon-only and phase-space kernels are built for it too.
 typedef void (*TransportKernel)(const TransportArgs);
+// Launches of one plan have their own (ONE) for the production, photon-only and
+// phase-space kernels.
 struct Variant {
     int max_threads, min_blocks;
-    bool prof, agg, sched, kerma, phsp;
+    bool prof, agg, sched, kerma, phsp, one;
     TransportKernel fn;
 };
 static const Variant kVariants[] = {
-    {512, 1, false, false, false, false, false, k_transport<512, 1, false, false, false, false, false>},
-    {384, 2, false, false, false, false, false, k_transport<384, 2, false, false, false, false, false>},
-    {1024, 1, false, false, false, false, false, k_transport<1024, 1, false, false, false, false, false>},
-    {1024, 1, true, false, false, false, false, k_transport<1024, 1, true, false, false, false, false>},
-    {1024, 1, false, true, false, false, false, k_transport<1024, 1, false, true, false, false, false>},
-    {1024, 1, false, false, true, false, false, k_transport<1024, 1, false, false, true, false, false>},
-    {1024, 1, false, false, false, true, false, k_transport<1024, 1, false, false, false, true, false>},
-    {1024, 1, false, false, false, false, true, k_transport<1024, 1, false, false, false, false, true>},
+    {512, 1, false, false, false, false, false, false, k_transport<512, 1, false, false, false, false, false, false>},
+    {384, 2, false, false, false, false, false, false, k_transport<384, 2, false, false, false, false, false, false>},
+    {1024, 1, false, false, false, false, false, true, k_transport<1024, 1, false, false, false, false, false, true>},
+    {1024, 1, false, false, false, false, false, false, k_transport<1024, 1, false, false, false, false, false, false>},
+    {1024, 1, true, false, false, false, false, false, k_transport<1024, 1, true, false, false, false, false, false>},
+    {1024, 1, false, true, false, false, false, false, k_transport<1024, 1, false, true, false, false, false, false>},
+    {1024, 1, false, false, true, false, false, false, k_transport<1024, 1, false, false, true, false, false, false>},
+    {1024, 1, false, false, false, true, false, true, k_transport<1024, 1, false, false, false, true, false, true>},
+    {1024, 1, false, false, false, true, false, false, k_transport<1024, 1, false, false, false, true, false, false>},
+    {1024, 1, false, false, false, false, true, true, k_transport<1024, 1, false, false, false, false, true, true>},
+    {1024, 1, false, false, false, false, true, false, k_transport<1024, 1, false, false, false, false, true, false>},
 };
 
 // The first variant (most registers first) whose bound covers the launch.
 static TransportKernel pick_variant(int block, int blocks_per_sm, bool prof, bool agg, bool sched, bool kerma,
-                                    bool phsp) {
+                                    bool phsp, bool one) {
     for (const Variant &v : kVariants)
         if (v.prof == prof && v.agg == agg && v.sched == sched && v.kerma == kerma && v.phsp == phsp &&
+            (one || !v.one) &&
             block <= v.max_threads && block * blocks_per_sm <= v.max_threads * v.min_blocks)
             return v.fn;
     return nullptr;
@@ -1267,7 +1299,7 @@ cudaError_t transport_configure() {
 const void *transport_kernel(const TransportArgs &a, int block, int blocks_per_sm) {
     return (const void *)pick_variant(block, blocks_per_sm, (a.flags & GPUMCD_LAUNCH_PROFILE) != 0u,
                                       (a.flags & GPUMCD_LAUNCH_WARP_AGGREGATE) != 0u, a.refill_period != 1u,
-                                      (a.flags & GPUMCD_LAUNCH_KERMA) != 0u, a.phsp != 0u);
+                                      (a.flags & GPUMCD_LAUNCH_KERMA) != 0u, a.phsp != 0u, a.n_plans == 1);
 }
 
 cudaError_t launch_transport(const TransportArgs &a, int grid, int block, int blocks_per_sm, cudaStream_t s) {
@@ -1314,7 +1346,7 @@ __device__ __forceinline__ int group_key(const PlanDev &P, unsigned long long h)
     p.lin_hi = 0u;
     p.draw = 0u;
     p.plan = 0u;
-    const uint4 r = draw4(p, P);
+    const uint4 r = philox4x32_10(make_uint4(p.draw, p.lin_lo, p.lin_hi, p.hist), make_uint2(P.key_lo, P.key_hi));
     const float z = u01(r.z);
     const float *cdf = P.spec;
     int lo = 0, hi = P.n_spec - 1;  // first bin with cdf[i+1] >= z, as sample_spectrum finds it
@@ -1440,8 +1472,8 @@ __global__ void k_debug_sample(const float *tabg, Phys ph, int kind, float p0, i
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     PlanDev P{};
-    P.key_lo = (uint32_t)seed;
-    P.key_hi = (uint32_t)(seed >> 32);
+    const uint2 k = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
+    const auto key = [k](int r) { return philox_round_key(k, r); };
     P.spec = spec;
     P.n_spec = n_spec;
     Lane p;
@@ -1455,22 +1487,22 @@ __global__ void k_debug_sample(const float *tabg, Phys ph, int kind, float p0, i
     unsigned capped = 0;
     if (kind == 0 || kind == 6) {
         float c;
-        const float eps = sample_kn(p, P, p0 / kMC2f, &c, &wd, &capped);
+        const float eps = sample_kn(p, key, p0 / kMC2f, &c, &wd, &capped);
         v = kind == 0 ? c : eps;
     } else if (kind == 1) {
-        v = sample_sauter(p, P, p0, &wd, &capped);
+        v = sample_sauter(p, key, p0, &wd, &capped);
     } else if (kind == 2) {
-        v = sample_hard(p, P, true, p0, ph.t_c, 0.f, 0.f, &wd, &capped);
+        v = sample_hard(p, key, true, p0, ph.t_c, 0.f, 0.f, &wd, &capped);
     } else if (kind == 3) {
-        v = sample_hard(p, P, false, p0, ph.k_c, __ldg(tabg + TAB_BREM + 2 * material),
+        v = sample_hard(p, key, false, p0, ph.k_c, __ldg(tabg + TAB_BREM + 2 * material),
                         __ldg(tabg + TAB_BREM + 2 * material + 1), &wd, &capped);
     } else if (kind == 4) {
         // the transport's own ms_mu, given the tables in global memory instead
         // of their shared-memory copy (the same word of the draw as a step uses)
-        const uint4 r = draw4(p, P);
+        const uint4 r = draw4(p, key);
         v = ms_mu(tabg, ph.grid, p0, u01(r.z));
     } else if (kind == 5) {
-        const uint4 r = draw4(p, P);
+        const uint4 r = draw4(p, key);
         v = sample_spectrum(P, u01(r.z));
     }
     out[i] = capped ? __int_as_float(0x7fc00000) : v;  // a capped draw shows up as NaN
