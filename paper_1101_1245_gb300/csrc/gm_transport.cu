@@ -47,7 +47,8 @@ struct WarpState {
 
 struct Lane {
     float x, y, z, ux, uy, uz;
-    uint32_t E, hist, lin_lo, lin_hi, draw, plan;
+    uint32_t E, hist, draw, plan;
+    PhiloxLineage lin;
     bool act;
 };
 
@@ -104,15 +105,17 @@ struct RoundKeys {
 
 template <class Keys>
 __device__ __forceinline__ uint4 draw4(Lane &p, const Keys &key) {
-    const uint4 r = philox4x32_10_keyed(make_uint4(p.draw, p.lin_lo, p.lin_hi, p.hist), key);
+    const uint4 r = philox4x32_10_lineage(p.draw, p.hist, p.lin, key);
     ++p.draw;
     return r;
 }
 
 // Lineage of the j-th particle a parent creates at draw index `draw`: a 64-bit
 // finalizer of (parent lineage, draw, j), never equal to the primary's lineage 1.
-__device__ __forceinline__ void child_lineage(const Lane &p, uint32_t j, uint32_t &lo, uint32_t &hi) {
-    unsigned long long z = ((unsigned long long)p.lin_hi << 32) | p.lin_lo;
+template <class Keys>
+__device__ __forceinline__ void child_lineage(const Lane &p, uint32_t j, const Keys &key, uint32_t &lo, uint32_t &hi) {
+    const uint2 own = philox_lineage_words(p.lin.a, p.lin.c, key(0), key(1));
+    unsigned long long z = ((unsigned long long)own.y << 32) | own.x;
     z ^= ((unsigned long long)p.draw << 20) ^ ((unsigned long long)(j + 1) << 52) ^ 0x9E3779B97F4A7C15ull;
     z = (z ^ (z >> 33)) * 0xFF51AFD7ED558CCDull;
     z = (z ^ (z >> 33)) * 0xC4CEB9FE1A85EC53ull;
@@ -227,33 +230,37 @@ __device__ __forceinline__ void rotate(float &ux, float &uy, float &uz, float c,
 
 // Push a new particle onto the warp's private stack of its type (headroom is
 // guaranteed by the caller before each step).
+template <bool ONE>
 __device__ __forceinline__ void push(const TransportArgs &A, const Smem &S, int gw, int w, int type,
                                      float x, float y, float z, float ux, float uy, float uz,
                                      uint32_t E, const Lane &parent, uint32_t j) {
     uint32_t lo, hi;
-    child_lineage(parent, j, lo, hi);
+    const RoundKeys<ONE> key{A, S.plans[parent.plan]};
+    child_lineage(parent, j, key, lo, hi);
+    const PhiloxLineage lin = philox_lineage(lo, hi, key(0), key(1));
     const unsigned slot = atomicAdd(&S.ws[w].stk[type], 1u);
     Rec *r = A.stacks + ((size_t)gw * 2 + type) * A.stack_cap + slot;
     r->a = make_float4(x, y, z, ux);
     r->b = make_float4(uy, uz, __uint_as_float(E), __uint_as_float(parent.hist));
-    r->c = make_uint4(lo, hi, 0u, parent.plan);
+    r->c = make_uint4(lin.a, lin.c, 0u, parent.plan);
     count(S, w, type == 0 ? CNT_PHOTONS : CNT_ELECTRONS);
 }
 
 // An electron set in motion by a photon: pushed for transport, or, in the
 // photon-only mode (GPUMCD_LAUNCH_KERMA), deposited in the voxel `idx` of the
 // photon's interaction.
-template <bool KERMA>
+template <bool KERMA, bool ONE>
 __device__ __forceinline__ void emit_electron(const TransportArgs &A, const Smem &S, int gw, int w,
                                               const PlanDev &P, uint32_t idx, float vx, float vy, float vz,
                                               uint32_t E, const Lane &parent, uint32_t j) {
     if (KERMA)
         deposit(P, parent.hist, idx, E);
     else
-        push(A, S, gw, w, 1, parent.x, parent.y, parent.z, vx, vy, vz, E, parent, j);
+        push<ONE>(A, S, gw, w, 1, parent.x, parent.y, parent.z, vx, vy, vz, E, parent, j);
 }
 
-__device__ __forceinline__ void load_rec(Lane &p, const Rec &r) {
+template <bool ONE>
+__device__ __forceinline__ void load_rec(const TransportArgs &A, const Smem &S, Lane &p, const Rec &r) {
     const float4 a = r.a;
     const float4 b = r.b;
     const uint4 c = r.c;
@@ -261,7 +268,10 @@ __device__ __forceinline__ void load_rec(Lane &p, const Rec &r) {
     p.uy = b.x; p.uz = b.y; p.E = __float_as_uint(b.z); p.hist = __float_as_uint(b.w);
     // the plan field indexes the CTA's 64-entry plan table, all of whose
     // entries are set at launch: masked, it stays in range by construction
-    p.lin_lo = c.x; p.lin_hi = c.y; p.draw = c.z; p.plan = c.w & (GPUMCD_MAX_PLANS_PER_RUN - 1);
+    p.draw = c.z; p.plan = c.w & (GPUMCD_MAX_PLANS_PER_RUN - 1);
+    p.lin.a = c.x;
+    p.lin.b = philox_lineage_b(c.y, RoundKeys<ONE>{A, S.plans[p.plan]}(1));
+    p.lin.c = c.y;
     p.act = true;
 }
 
@@ -269,7 +279,7 @@ __device__ __forceinline__ Rec make_rec(const Lane &p) {
     Rec r;
     r.a = make_float4(p.x, p.y, p.z, p.ux);
     r.b = make_float4(p.uy, p.uz, __uint_as_float(p.E), __uint_as_float(p.hist));
-    r.c = make_uint4(p.lin_lo, p.lin_hi, p.draw, p.plan);
+    r.c = make_uint4(p.lin.a, p.lin.c, p.draw, p.plan);
     return r;
 }
 
@@ -408,12 +418,12 @@ __device__ __forceinline__ float sample_spectrum(const PlanDev &P, float z) {
 // claims (refill), not the sample.
 template <bool PHSP, bool ONE>
 __device__ __forceinline__ uint32_t make_primary(const TransportArgs &A, Lane &p, const PlanDev &P, uint32_t plan, uint64_t h) {
+    const RoundKeys<ONE> key{A, P};
     p.hist = (uint32_t)h;
-    p.lin_lo = 1u;
-    p.lin_hi = 0u;
+    p.lin = philox_lineage(1u, 0u, key(0), key(1));
     p.draw = 0u;
     p.plan = plan;
-    const uint4 r = draw4(p, RoundKeys<ONE>{A, P});
+    const uint4 r = draw4(p, key);
     if (PHSP && P.beam == GPUMCD_BEAM_PHASE_SPACE) {
         const float4 *ps = reinterpret_cast<const float4 *>(P.spec);
         const uint32_t k = (uint32_t)(h % (unsigned long long)P.n_phsp);
@@ -521,7 +531,7 @@ __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Sm
             const float e1f = (float)e1 * kQf;
             float ex = E * p.ux - e1f * vx, ey = E * p.uy - e1f * vy, ez = E * p.uz - e1f * vz;
             const float n = rsqrtf(fmaxf(ex * ex + ey * ey + ez * ez, 1e-30f));
-            emit_electron<KERMA>(A, S, gw, w, P, idx, ex * n, ey * n, ez * n, te, p, 0);
+            emit_electron<KERMA, ONE>(A, S, gw, w, P, idx, ex * n, ey * n, ez * n, te, p, 0);
         } else {
             deposit(P, p.hist, idx, te);
         }
@@ -546,7 +556,7 @@ __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Sm
             const float sn = sqrtf(fmaxf(0.0f, (1.0f - c) * (1.0f + c)));
             float vx = p.ux, vy = p.uy, vz = p.uz;
             rotate(vx, vy, vz, c, sn, cp, sp);
-            emit_electron<KERMA>(A, S, gw, w, P, idx, vx, vy, vz, p.E, p, 0);
+            emit_electron<KERMA, ONE>(A, S, gw, w, P, idx, vx, vy, vz, p.E, p, 0);
         } else {
             deposit(P, p.hist, idx, p.E);
         }
@@ -571,7 +581,7 @@ __device__ __forceinline__ void photon_interact(const TransportArgs &A, const Sm
                 __sincosf(th, &st, &ct);
                 float vx = p.ux, vy = p.uy, vz = p.uz;
                 rotate(vx, vy, vz, ct, st, j == 0 ? cp : -cp, j == 0 ? sp : -sp);
-                emit_electron<KERMA>(A, S, gw, w, P, idx, vx, vy, vz, te, p, (uint32_t)j);
+                emit_electron<KERMA, ONE>(A, S, gw, w, P, idx, vx, vy, vz, te, p, (uint32_t)j);
             } else {
                 deposit(P, p.hist, idx, te);
             }
@@ -740,7 +750,7 @@ __device__ __forceinline__ void hard_event(const TransportArgs &A, const Smem &S
     float vx = p.ux, vy = p.uy, vz = p.uz;
     rotate(vx, vy, vz, c, sn, cp, sp);
     if (e2 >= (moller ? ph.e_abs_q : ph.p_cut_q))
-        push(A, S, gw, w, moller ? 1 : 0, p.x, p.y, p.z, vx, vy, vz, e2, p, 0);
+        push<ONE>(A, S, gw, w, moller ? 1 : 0, p.x, p.y, p.z, vx, vy, vz, e2, p, 0);
     else
         deposit(P, p.hist, idx1, e2);
     if (moller) rotate(p.ux, p.uy, p.uz, c2, sqrtf(fmaxf(0.f, 1.f - c2 * c2)), -cp, -sp);
@@ -836,7 +846,7 @@ __device__ int refill(const TransportArgs &A, const Smem &S, CtaFlags &F, Lane &
         if (take) {
             const unsigned rank = __popc(empty & lt);
             if (!p.act && rank < take)
-                load_rec(p, A.stacks[((size_t)gw * 2 + t) * A.stack_cap + (sc - 1u - rank)]);
+                load_rec<ONE>(A, S, p, A.stacks[((size_t)gw * 2 + t) * A.stack_cap + (sc - 1u - rank)]);
             __syncwarp();
             if (lane == 0) ws.stk[t] = sc - take;
             __syncwarp();
@@ -859,7 +869,7 @@ __device__ int refill(const TransportArgs &A, const Smem &S, CtaFlags &F, Lane &
         }
         const unsigned take = (unsigned)min((unsigned long long)__popc(empty), hi - lo);
         const unsigned rank = __popc(empty & lt);
-        if (!p.act && rank < take) load_rec(p, A.in[t].rec[lo + rank]);
+        if (!p.act && rank < take) load_rec<ONE>(A, S, p, A.in[t].rec[lo + rank]);
         __syncwarp();
         if (lane == 0) {
             ws.q_lo[t] = lo + take;
@@ -984,7 +994,7 @@ __device__ __forceinline__ void hard_pass(const TransportArgs &A, const Smem &S,
     uint32_t idx1 = 0u;
     if ((unsigned)lane < take) {
         const HardRec &h = A.hard[(size_t)gw * HARD_CAP + (hc - 1u - lane)];
-        load_rec(p, h.r);
+        load_rec<ONE>(A, S, p, h.r);
         sig_hat = h.sig_hat;
         idx1 = h.idx;
     }
@@ -1097,7 +1107,8 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
     Lane p;
     p.act = false;
     p.x = p.y = p.z = p.ux = p.uy = p.uz = 0.f;
-    p.E = p.hist = p.lin_lo = p.lin_hi = p.draw = p.plan = 0;
+    p.E = p.hist = p.draw = p.plan = 0;
+    p.lin = PhiloxLineage{0u, 0u, 0u};
     constexpr bool agg = AGG;
     constexpr bool prof = PROF;
     // start on the type that has work (electron-beam launches start on electrons)
@@ -1340,13 +1351,8 @@ __device__ __forceinline__ int group_key(const PlanDev &P, unsigned long long h)
         const int b = (int)(__float_as_uint(E) >> 17) - ((127 - 10) << 6);
         return PHSP_GROUP_BINS - 1 - min(max(b, 0), PHSP_GROUP_BINS - 1);
     }
-    Lane p;
-    p.hist = (uint32_t)h;
-    p.lin_lo = 1u;
-    p.lin_hi = 0u;
-    p.draw = 0u;
-    p.plan = 0u;
-    const uint4 r = philox4x32_10(make_uint4(p.draw, p.lin_lo, p.lin_hi, p.hist), make_uint2(P.key_lo, P.key_hi));
+    // draw 0 of the primary's lineage 1
+    const uint4 r = philox4x32_10(make_uint4(0u, 1u, 0u, (uint32_t)h), make_uint2(P.key_lo, P.key_hi));
     const float z = u01(r.z);
     const float *cdf = P.spec;
     int lo = 0, hi = P.n_spec - 1;  // first bin with cdf[i+1] >= z, as sample_spectrum finds it
@@ -1478,8 +1484,7 @@ __global__ void k_debug_sample(const float *tabg, Phys ph, int kind, float p0, i
     P.n_spec = n_spec;
     Lane p;
     p.hist = (uint32_t)i;
-    p.lin_lo = (uint32_t)(i >> 32);
-    p.lin_hi = 0x5EEDu;
+    p.lin = philox_lineage((uint32_t)(i >> 32), 0x5EEDu, key(0), key(1));
     p.draw = 0;
     p.plan = 0;
     float v = 0.f;
