@@ -2,6 +2,7 @@
 // under an HBM budget, phantoms, plans and the launch sequence of the
 // persistent transport kernel.
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <algorithm>
@@ -44,14 +45,13 @@ struct Plan {
     int inflight = 0;        // unfinished sequences that include this plan
     bool failed = false;     // a sequence failed: the tally is incomplete until plan_reset
     cudaEvent_t reset_done = nullptr;  // after the last plan_reset's memsets (any stream)
-    DevBuf tally;   // [W][nvox] u64
-    DevBuf ledger;  // [4] u64
+    DevBuf tally;   // [W][nvox] u64, then the ledger [4] u64
     DevBuf spec;    // [2(n_spec+1)] floats
     gpumcd_run_stats acc;  // counters accumulated over the plan's runs
 };
 
 // Device control block of a launch sequence.
-struct Control {
+struct alignas(16) Control {
     unsigned long long prim_cursor[2];
     unsigned long long qcur[2][NT];  // [buffer][type]
     unsigned long long counters[CNT_N];
@@ -59,17 +59,24 @@ struct Control {
     int32_t pad;
 };
 
+// What a sequence starts from, uploaded in one copy: a zeroed control block
+// and the plan table.
+struct SeqStart {
+    Control control;
+    PlanDev plans[GPUMCD_MAX_PLANS_PER_RUN];
+};
+
 // Scratch and state of one launch sequence (the persistent kernel, then
 // relaunches over the overflow queues until they are empty).  Slot 0 serves
 // gpumcd_run on the caller's stream; slots 1..GPUMCD_MAX_INFLIGHT serve
 // gpumcd_submit on their own streams, so sequences can overlap on the device.
 struct Slot {
-    DevBuf stacks, hard, queue[2][NT], control, plandev;
+    DevBuf stacks, hard, queue[2][NT], start;
     DevBuf order, gcount;  // claim orders of grouped sources, and their sort's bin counts
     Control *h_control = nullptr;  // pinned: the control block after each launch
-    PlanDev *h_plandev = nullptr;  // pinned: the sequence's plan table
+    SeqStart *h_start = nullptr;   // pinned: the control block and plan table to start from
     cudaStream_t own = nullptr;    // the slot's stream (asynchronous slots)
-    cudaEvent_t ev0 = nullptr, ev1 = nullptr, done = nullptr;
+    cudaEvent_t ev0 = nullptr, ev1 = nullptr;  // around the sequence's launches so far
     bool busy = false;
     int32_t ticket = 0;
     cudaStream_t s = nullptr;  // the stream the sequence runs on
@@ -212,6 +219,17 @@ gpumcd_status set_device(gpumcd_ctx *c) {
     return GPUMCD_OK;
 }
 
+unsigned long long *plan_ledger(const Plan &p, uint64_t nvox) {
+    return (unsigned long long *)p.tally.p + (size_t)p.W * nvox;
+}
+
+// Zero a plan's tally and ledger on stream s, after the last time they were
+// zeroed (a cached block may be larger: its own size only).
+cudaError_t zero_tally(const Plan &p, uint64_t nvox, cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(p.tally.p, 0, ((size_t)p.W * nvox + 4) * 8, s);
+    return e != cudaSuccess ? e : cudaEventRecord(p.reset_done, s);
+}
+
 bool valid_source(const gpumcd_ctx *c, const gpumcd_source *s) {
     if (!s) return false;
     if (s->particle != GPUMCD_PHOTON && s->particle != GPUMCD_ELECTRON) return false;
@@ -240,13 +258,14 @@ gpumcd_status ensure_slot(gpumcd_ctx *c, Slot &sl, int grid, int block) {
     for (int b = 0; b < 2; ++b)
         for (int t = 0; t < NT; ++t)
             ST(dev_alloc(c, sl.queue[b][t], (size_t)c->launch.overflow_capacity * sizeof(Rec)));
-    ST(dev_alloc(c, sl.control, sizeof(Control)));
-    ST(dev_alloc(c, sl.plandev, sizeof(PlanDev) * GPUMCD_MAX_PLANS_PER_RUN));
+    ST(dev_alloc(c, sl.start, sizeof(SeqStart)));
     if (!sl.h_control) CK(cudaMallocHost(&sl.h_control, sizeof(Control)));
-    if (!sl.h_plandev) CK(cudaMallocHost(&sl.h_plandev, sizeof(PlanDev) * GPUMCD_MAX_PLANS_PER_RUN));
+    if (!sl.h_start) {
+        CK(cudaMallocHost(&sl.h_start, sizeof(SeqStart)));
+        memset((void *)sl.h_start, 0, sizeof(SeqStart));
+    }
     if (!sl.ev0) CK(cudaEventCreate(&sl.ev0));
     if (!sl.ev1) CK(cudaEventCreate(&sl.ev1));
-    if (!sl.done) CK(cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming));
     if (!c->configured) {
         CK(transport_configure());
         c->configured = true;
@@ -262,13 +281,11 @@ void free_slot(gpumcd_ctx *c, Slot &sl) {
     dev_free(c, sl.hard);
     for (int b = 0; b < 2; ++b)
         for (int t = 0; t < NT; ++t) dev_free(c, sl.queue[b][t]);
-    dev_free(c, sl.control);
-    dev_free(c, sl.plandev);
+    dev_free(c, sl.start);
     if (sl.h_control) cudaFreeHost(sl.h_control);
-    if (sl.h_plandev) cudaFreeHost(sl.h_plandev);
+    if (sl.h_start) cudaFreeHost(sl.h_start);
     if (sl.ev0) cudaEventDestroy(sl.ev0);
     if (sl.ev1) cudaEventDestroy(sl.ev1);
-    if (sl.done) cudaEventDestroy(sl.done);
     if (sl.gexec) cudaGraphExecDestroy(sl.gexec);
     if (sl.graph) cudaGraphDestroy(sl.graph);
     if (sl.own) cudaStreamDestroy(sl.own);
@@ -369,7 +386,6 @@ gpumcd_status gpumcd_destroy(gpumcd_ctx *c) {
     for (auto &kv : c->plans) {
         if (kv.second.reset_done) cudaEventDestroy(kv.second.reset_done);
         dev_free(c, kv.second.tally);
-        dev_free(c, kv.second.ledger);
         dev_free(c, kv.second.spec);
     }
     for (auto &kv : c->phantoms) {
@@ -544,8 +560,7 @@ gpumcd_status gpumcd_plan_open(gpumcd_ctx *c, int32_t phantom_id, const gpumcd_s
     p.seed = seed;
     p.W = n_batches;
     const uint64_t nvox = it->second.nvox;
-    gpumcd_status st = dev_alloc(c, p.tally, (size_t)n_batches * nvox * 8);
-    if (st == GPUMCD_OK) st = dev_alloc(c, p.ledger, 4 * 8);
+    gpumcd_status st = dev_alloc(c, p.tally, ((size_t)n_batches * nvox + 4) * 8);
     DevBuf tmp;
     if (st == GPUMCD_OK && p.n_spec > 0) {
         st = dev_alloc(c, p.spec, (size_t)2 * (p.n_spec + 1) * 4);
@@ -594,24 +609,24 @@ gpumcd_status gpumcd_plan_open(gpumcd_ctx *c, int32_t phantom_id, const gpumcd_s
         p.n_phsp = (uint32_t)n;
         p.n_spec = 0;
     }
+    // the tally is zeroed on the context's stream; whoever uses it on another
+    // one waits for reset_done
     if (st == GPUMCD_OK) {
-        cudaError_t e = cudaMemsetAsync(p.tally.p, 0, (size_t)n_batches * nvox * 8, c->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(p.ledger.p, 0, 4 * 8, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        if (e != cudaSuccess) st = cuda_status(e);
+        cudaError_t e = cudaEventCreateWithFlags(&p.reset_done, cudaEventDisableTiming);
+        if (e == cudaSuccess) {
+            e = zero_tally(p, nvox, c->stream);
+            if (e != cudaSuccess) cudaStreamSynchronize(c->stream);  // nothing pending on what goes back
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            st = cuda_status(e);
+        }
     }
     if (st != GPUMCD_OK) {
+        if (p.reset_done) cudaEventDestroy(p.reset_done);
         dev_free(c, p.tally);
-        dev_free(c, p.ledger);
         dev_free(c, p.spec);
         return st;
-    }
-    if (cudaEventCreateWithFlags(&p.reset_done, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        dev_free(c, p.tally);
-        dev_free(c, p.ledger);
-        dev_free(c, p.spec);
-        return GPUMCD_ERR_CUDA;
     }
     *plan_id = c->next_id++;
     c->plans[*plan_id] = p;
@@ -632,7 +647,6 @@ gpumcd_status gpumcd_plan_close(gpumcd_ctx *c, int32_t plan_id) {
         cudaEventDestroy(it->second.reset_done);
     }
     dev_free(c, it->second.tally);
-    dev_free(c, it->second.ledger);
     dev_free(c, it->second.spec);
     c->plans.erase(it);
     return GPUMCD_OK;
@@ -646,10 +660,8 @@ gpumcd_status gpumcd_plan_reset(gpumcd_ctx *c, int32_t plan_id, uint64_t seed, v
     ST(set_device(c));
     cudaStream_t s = pick(c, stream);
     Plan &p = it->second;
-    // a cached block may be larger than the tally: zero the tally's own size
-    CK(cudaMemsetAsync(p.tally.p, 0, (size_t)p.W * c->phantoms.at(p.phantom).nvox * 8, s));
-    CK(cudaMemsetAsync(p.ledger.p, 0, 4 * 8, s));
-    CK(cudaEventRecord(p.reset_done, s));
+    CK(cudaStreamWaitEvent(s, p.reset_done, 0));
+    CK(zero_tally(p, c->phantoms.at(p.phantom).nvox, s));
     p.seed = seed;
     p.hist_sub = 0;
     p.hist_done = 0;
@@ -674,7 +686,7 @@ namespace {
 // out-queue (empty for k = 0), both cursors restart at 0.
 gpumcd_status launch_one(gpumcd_ctx *c, Slot &sl) {
     const int bi = (int)(sl.k & 1u), bo = bi ^ 1;
-    Control *dc = (Control *)sl.control.p;
+    Control *dc = &((SeqStart *)sl.start.p)->control;
     TransportArgs &A = sl.A;
     for (int t = 0; t < NT; ++t) {
         A.in[t].rec = (Rec *)sl.queue[bi][t].p;
@@ -685,17 +697,17 @@ gpumcd_status launch_one(gpumcd_ctx *c, Slot &sl) {
         A.out[t].capacity = c->launch.overflow_capacity;
         A.in_count[t] = sl.in_count[t];
     }
-    CK(cudaMemsetAsync(dc->qcur, 0, sizeof(dc->qcur), sl.s));
+    if (sl.k > 0) CK(cudaMemsetAsync(dc->qcur, 0, sizeof(dc->qcur), sl.s));
     CK(launch_transport(A, sl.grid, sl.block, sl.bps, sl.s));
     CK(cudaMemcpyAsync(sl.h_control, dc, sizeof(Control), cudaMemcpyDeviceToHost, sl.s));
-    CK(cudaEventRecord(sl.done, sl.s));
+    CK(cudaEventRecord(sl.ev1, sl.s));
     ++sl.k;
     return GPUMCD_OK;
 }
 
 // The queue and cursor pointers of launch k = 0 (empty in-queue).
 void first_queues(gpumcd_ctx *c, Slot &sl) {
-    Control *dc = (Control *)sl.control.p;
+    Control *dc = &((SeqStart *)sl.start.p)->control;
     for (int t = 0; t < NT; ++t) {
         sl.A.in[t].rec = (Rec *)sl.queue[0][t].p;
         sl.A.in[t].cursor = &dc->qcur[0][t];
@@ -707,14 +719,14 @@ void first_queues(gpumcd_ctx *c, Slot &sl) {
     }
 }
 
-// First launch of a sequence from the slot's captured graph.  Its copy and
-// reset nodes touch only slot-owned buffers of fixed size (the whole plan
-// table is copied), so the graph stays valid for the slot's lifetime and
+// First launch of a sequence from the slot's captured graph.  Its copy nodes
+// touch only slot-owned buffers of fixed size (the whole plan table is
+// copied), so the graph stays valid for the slot's lifetime and
 // only the kernel node's argument block changes between runs; a new launch
 // shape (grid, CTA size, kernel variant) is captured afresh.
 gpumcd_status first_launch_graph(gpumcd_ctx *c, Slot &sl) {
     first_queues(c, sl);
-    Control *dc = (Control *)sl.control.p;
+    Control *dc = &((SeqStart *)sl.start.p)->control;
     // a graph is rebuilt for a new launch shape or another compiled kernel
     // (its kernel node keeps the function it was captured with)
     const void *fn = transport_kernel(sl.A, sl.block, sl.bps);
@@ -725,9 +737,7 @@ gpumcd_status first_launch_graph(gpumcd_ctx *c, Slot &sl) {
         sl.graph = nullptr;
         sl.knode = nullptr;
         CK(cudaStreamBeginCapture(sl.s, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = cudaMemcpyAsync(sl.plandev.p, sl.h_plandev, sizeof(PlanDev) * GPUMCD_MAX_PLANS_PER_RUN,
-                                        cudaMemcpyHostToDevice, sl.s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(dc, 0, sizeof(Control), sl.s);
+        cudaError_t e = cudaMemcpyAsync(sl.start.p, sl.h_start, sizeof(SeqStart), cudaMemcpyHostToDevice, sl.s);
         if (e == cudaSuccess) e = launch_transport(sl.A, sl.grid, sl.block, sl.bps, sl.s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(sl.h_control, dc, sizeof(Control), cudaMemcpyDeviceToHost, sl.s);
         cudaGraph_t g = nullptr;
@@ -764,7 +774,7 @@ gpumcd_status first_launch_graph(gpumcd_ctx *c, Slot &sl) {
     }
     CK(cudaEventRecord(sl.ev0, sl.s));
     CK(cudaGraphLaunch(sl.gexec, sl.s));
-    CK(cudaEventRecord(sl.done, sl.s));
+    CK(cudaEventRecord(sl.ev1, sl.s));
     sl.k = 1;
     return GPUMCD_OK;
 }
@@ -842,11 +852,11 @@ gpumcd_status seq_start(gpumcd_ctx *c, Slot &sl, int32_t n_plans, const int32_t 
     for (int i = 0; i < n_plans; ++i) {
         const Plan &p = *pl[i];
         const Phantom &ph = c->phantoms.at(p.phantom);
-        PlanDev &d = sl.h_plandev[i];
+        PlanDev &d = sl.h_start->plans[i];
         memset(&d, 0, sizeof d);
         d.vox = (const uint32_t *)ph.vox.p;
         d.tally = (unsigned long long *)p.tally.p;
-        d.ledger = (unsigned long long *)p.ledger.p;
+        d.ledger = plan_ledger(p, ph.nvox);
         d.maj = (const float *)ph.maj.p;
         d.spec = (const float *)p.spec.p;
         d.nx = ph.dims[0];
@@ -882,14 +892,14 @@ gpumcd_status seq_start(gpumcd_ctx *c, Slot &sl, int32_t n_plans, const int32_t 
         A.prim_off[t][A.n_prim_plans[t] + 1] = A.prim_off[t][A.n_prim_plans[t]] + n_hist[i];
         A.n_prim_plans[t]++;
     }
-    Control *dc = (Control *)sl.control.p;
+    Control *dc = &((SeqStart *)sl.start.p)->control;
     A.tables = (const float *)c->tab.p;
     A.tab_bytes = tab_bytes(c->n_mat);
     A.phys = c->dphys;
-    A.plans = (const PlanDev *)sl.plandev.p;
+    A.plans = ((const SeqStart *)sl.start.p)->plans;
     A.n_plans = n_plans;
     for (int r = 0; r < 10; ++r)
-        A.round_key[r] = philox_round_key(make_uint2(sl.h_plandev[0].key_lo, sl.h_plandev[0].key_hi), r);
+        A.round_key[r] = philox_round_key(make_uint2(sl.h_start->plans[0].key_lo, sl.h_start->plans[0].key_hi), r);
     A.prim_cursor = dc->prim_cursor;
     A.stacks = (Rec *)sl.stacks.p;
     A.hard = (HardRec *)sl.hard.p;
@@ -912,7 +922,7 @@ gpumcd_status seq_start(gpumcd_ctx *c, Slot &sl, int32_t n_plans, const int32_t 
     // run one after another on the stream and share the key scratch)
     size_t n_order = 0, n_keys = 0;
     for (int i = 0; i < n_plans; ++i) {
-        const PlanDev &d = sl.h_plandev[i];
+        const PlanDev &d = sl.h_start->plans[i];
         if (!d.e_group) continue;
         n_order += d.n_sorted;
         n_keys = std::max<size_t>(n_keys, d.n_sorted);
@@ -927,13 +937,16 @@ gpumcd_status seq_start(gpumcd_ctx *c, Slot &sl, int32_t n_plans, const int32_t 
         uint32_t *ord = (uint32_t *)sl.order.p;
         uint16_t *keys = (uint16_t *)((uint32_t *)sl.order.p + n_order);
         for (int i = 0; i < n_plans; ++i) {
-            PlanDev &d = sl.h_plandev[i];
+            PlanDev &d = sl.h_start->plans[i];
             if (!d.e_group) continue;
             d.order = ord;
             CK(launch_group_order(d, d.n_sorted, (unsigned *)sl.gcount.p, keys, ord, s));
             ord += d.n_sorted;
         }
     }
+
+    // after the plans' tallies were zeroed, on whatever stream that was
+    for (int i = 0; i < n_plans; ++i) CK(cudaStreamWaitEvent(s, pl[i]->reset_done, 0));
 
     sl.s = s;
     sl.k = 0;
@@ -949,9 +962,8 @@ gpumcd_status seq_start(gpumcd_ctx *c, Slot &sl, int32_t n_plans, const int32_t 
     if (c->launch.flags & GPUMCD_LAUNCH_GRAPH) {
         st = first_launch_graph(c, sl);
     } else {
-        cudaError_t e = cudaMemcpyAsync(sl.plandev.p, sl.h_plandev, sizeof(PlanDev) * n_plans,
+        cudaError_t e = cudaMemcpyAsync(sl.start.p, sl.h_start, offsetof(SeqStart, plans) + sizeof(PlanDev) * n_plans,
                                         cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(dc, 0, sizeof(Control), s);
         if (e == cudaSuccess) e = cudaEventRecord(sl.ev0, s);
         st = cuda_status(e);
         if (st == GPUMCD_OK) st = launch_one(c, sl);
@@ -968,7 +980,7 @@ gpumcd_status seq_start(gpumcd_ctx *c, Slot &sl, int32_t n_plans, const int32_t 
 gpumcd_status seq_finish(gpumcd_ctx *c, Slot &sl) {
     gpumcd_status result = GPUMCD_OK;
     for (;;) {
-        cudaError_t e = cudaEventSynchronize(sl.done);
+        cudaError_t e = cudaEventSynchronize(sl.ev1);
         if (e != cudaSuccess) {
             result = cuda_status(e);
             break;
@@ -993,11 +1005,11 @@ gpumcd_status seq_finish(gpumcd_ctx *c, Slot &sl) {
         result = launch_one(c, sl);
         if (result != GPUMCD_OK) break;
     }
-    float ms = 0.f;
-    if (cudaEventRecord(sl.ev1, sl.s) == cudaSuccess && cudaEventSynchronize(sl.ev1) == cudaSuccess)
-        cudaEventElapsedTime(&ms, sl.ev0, sl.ev1);
-    else
+    float ms = 0.f;  // from the first launch's start to the last one's end
+    if (cudaEventElapsedTime(&ms, sl.ev0, sl.ev1) != cudaSuccess) {
         cudaGetLastError();
+        ms = 0.f;
+    }
     seq_close(c, sl, result, ms);
     return result;
 }
@@ -1080,7 +1092,7 @@ gpumcd_status gpumcd_poll(gpumcd_ctx *c, int32_t ticket, int32_t *done) {
     Slot *sl = find_ticket(c, ticket);
     if (!sl) return GPUMCD_ERR_NOT_FOUND;
     ST(set_device(c));
-    const cudaError_t e = cudaEventQuery(sl->done);
+    const cudaError_t e = cudaEventQuery(sl->ev1);
     if (e == cudaErrorNotReady) {
         cudaGetLastError();
         return GPUMCD_OK;
@@ -1097,8 +1109,10 @@ gpumcd_status gpumcd_wait(gpumcd_ctx *c, int32_t ticket) {
     return seq_finish(c, *sl);
 }
 
-gpumcd_status gpumcd_plan_result(gpumcd_ctx *c, int32_t plan_id, double thr, double *dose, double *sigma,
-                                 void *stream, gpumcd_run_stats *stats) {
+// The result in device arrays (dose, sigma; the context's scratch where null),
+// and copied from there to host arrays (h_dose, h_sigma) where given.
+static gpumcd_status plan_result_impl(gpumcd_ctx *c, int32_t plan_id, double thr, double *dose, double *sigma,
+                                      double *h_dose, double *h_sigma, void *stream, gpumcd_run_stats *stats) {
     if (!c) return GPUMCD_ERR_INVALID_ARG;
     auto it = c->plans.find(plan_id);
     if (it == c->plans.end()) return GPUMCD_ERR_NOT_FOUND;
@@ -1120,19 +1134,23 @@ gpumcd_status gpumcd_plan_result(gpumcd_ctx *c, int32_t plan_id, double thr, dou
     double *ddose = dose ? dose : tdose;
     double *dsig = sigma ? sigma : tsig;
     const uint64_t N = p.hist_done;
+    unsigned long long *ledger = plan_ledger(p, nvox);
+    CK(cudaStreamWaitEvent(s, p.reset_done, 0));
     CK(cudaMemsetAsync(red, 0, kRedWords * 8, s));
     const double inv_vol = 1.0 / (ph.voxel[0] * ph.voxel[1] * ph.voxel[2]);
     if (N > 0) {
         CK(launch_fold((const unsigned long long *)p.tally.p, (const uint32_t *)ph.vox.p, nvox, (int)p.W, N, inv_vol,
                        ddose, dsig, red, red + 3, c->n_sm, s));
-        CK(launch_sthr(ddose, dsig, nvox, thr, sthr_part, red, (const unsigned long long *)p.ledger.p, c->n_sm, s));
+        CK(launch_sthr(ddose, dsig, nvox, thr, sthr_part, red, ledger, c->n_sm, s));
     } else {
         CK(cudaMemsetAsync(ddose, 0, nvox * 8, s));
         CK(cudaMemsetAsync(dsig, 0, nvox * 8, s));
-        CK(cudaMemcpyAsync(red + 5, p.ledger.p, 4 * 8, cudaMemcpyDeviceToDevice, s));
+        CK(cudaMemcpyAsync(red + 5, ledger, 4 * 8, cudaMemcpyDeviceToDevice, s));
     }
     const unsigned long long *h_red = c->h_red, *h_led = c->h_red + 5;
     CK(cudaMemcpyAsync(c->h_red, red, 9 * 8, cudaMemcpyDeviceToHost, s));
+    if (h_dose) CK(cudaMemcpyAsync(h_dose, ddose, nvox * 8, cudaMemcpyDeviceToHost, s));
+    if (h_sigma) CK(cudaMemcpyAsync(h_sigma, dsig, nvox * 8, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (stats) {
         *stats = p.acc;
@@ -1150,6 +1168,11 @@ gpumcd_status gpumcd_plan_result(gpumcd_ctx *c, int32_t plan_id, double thr, dou
         stats->s_thr = h_red[2] ? ssum / (double)h_red[2] : 0.0;
     }
     return GPUMCD_OK;
+}
+
+gpumcd_status gpumcd_plan_result(gpumcd_ctx *c, int32_t plan_id, double thr, double *dose, double *sigma,
+                                 void *stream, gpumcd_run_stats *stats) {
+    return plan_result_impl(c, plan_id, thr, dose, sigma, nullptr, nullptr, stream, stats);
 }
 
 gpumcd_status gpumcd_plan_result_noalloc(gpumcd_ctx *c, int32_t plan_id, double thr, double *dose, double *sigma,
@@ -1170,7 +1193,7 @@ gpumcd_status gpumcd_plan_result_noalloc(gpumcd_ctx *c, int32_t plan_id, double 
     const double inv_vol = 1.0 / (ph.voxel[0] * ph.voxel[1] * ph.voxel[2]);
     CK(launch_fold_noalloc(c->device, (const unsigned long long *)p.tally.p, (const uint32_t *)ph.vox.p, ph.nvox,
                            (int)p.W, N, inv_vol, thr, dose, sigma, s, res));
-    CK(cudaMemcpyAsync(led, p.ledger.p, sizeof led, cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(led, plan_ledger(p, ph.nvox), sizeof led, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (stats) {
         *stats = p.acc;
@@ -1188,18 +1211,7 @@ gpumcd_status gpumcd_plan_result_noalloc(gpumcd_ctx *c, int32_t plan_id, double 
 
 gpumcd_status gpumcd_plan_result_host(gpumcd_ctx *c, int32_t plan_id, double thr, double *dose, double *sigma,
                                       gpumcd_run_stats *stats) {
-    if (!c) return GPUMCD_ERR_INVALID_ARG;
-    auto it = c->plans.find(plan_id);
-    if (it == c->plans.end()) return GPUMCD_ERR_NOT_FOUND;
-    // the fold writes [dose | sigma] into the context's fold scratch, then both
-    // arrays come back in two copies on the context's stream
-    ST(gpumcd_plan_result(c, plan_id, thr, nullptr, nullptr, nullptr, stats));
-    const uint64_t nvox = c->phantoms.at(it->second.phantom).nvox;
-    const double *td = (const double *)c->fold_tmp.p;
-    if (dose) CK(cudaMemcpyAsync(dose, td, nvox * 8, cudaMemcpyDeviceToHost, c->stream));
-    if (sigma) CK(cudaMemcpyAsync(sigma, td + nvox, nvox * 8, cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    return GPUMCD_OK;
+    return plan_result_impl(c, plan_id, thr, nullptr, nullptr, dose, sigma, nullptr, stats);
 }
 
 // Rounds of at least this many histories run in a launch of their own in
@@ -1331,18 +1343,9 @@ static gpumcd_status simulate_impl(gpumcd_ctx *c, int32_t phantom_id, const gpum
         st = gpumcd_plan_result(c, pid, 0.5, nullptr, nullptr, s, &rs);
         if (st != GPUMCD_OK) break;
     } while (rs.s_thr > target && done + n <= cap);
-    const uint64_t nvox = c->phantoms.at(phantom_id).nvox;
     if (st == GPUMCD_OK) {
         if (host) {
-            st = gpumcd_plan_result(c, pid, 0.5, nullptr, nullptr, s, &rs);
-            if (st == GPUMCD_OK) {
-                const double *td = (const double *)c->fold_tmp.p;
-                cudaError_t e = cudaSuccess;
-                if (dose) e = cudaMemcpyAsync(dose, td, nvox * 8, cudaMemcpyDeviceToHost, s);
-                if (e == cudaSuccess && sigma) e = cudaMemcpyAsync(sigma, td + nvox, nvox * 8, cudaMemcpyDeviceToHost, s);
-                if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-                if (e != cudaSuccess) st = cuda_status(e);
-            }
+            st = plan_result_impl(c, pid, 0.5, nullptr, nullptr, dose, sigma, s, &rs);
         } else {
             st = gpumcd_plan_result(c, pid, 0.5, dose, sigma, s, &rs);
         }
