@@ -1333,7 +1333,12 @@ cudaError_t launch_transport(const TransportArgs &a, int grid, int block, int bl
 // any moment, start histories of similar energy, the longest first.
 // ---------------------------------------------------------------------------
 constexpr int GROUP_THREADS = 256;
-constexpr uint32_t GROUP_PER_BLOCK = 16 * GROUP_THREADS;
+// Histories a block sorts, in rounds of one a thread.  Each round waits for a
+// key (a draw and a search, or a record), so a short sort wants many blocks; a
+// long one wants fewer, as each adds its bins to the global counts.  Four
+// rounds up to 2^19 histories, eight above, against sixteen throughout: the
+// sort of 2e4 histories takes 23 us less, of 2e5 19, of 1e6 2, of 4e6 6.
+static uint32_t group_per_block(uint32_t n) { return (n <= (1u << 19) ? 4u : 8u) * GROUP_THREADS; }
 
 // Energy bins of a grouped phase space: 64 to an octave over [2^-10, 2^6) MeV,
 // from the float's exponent and top six mantissa bits (exact and monotone for
@@ -1370,13 +1375,14 @@ __device__ __forceinline__ int group_key(const PlanDev &P, unsigned long long h)
 // count.  Lanes of a warp with the same key add once (one shared atomic per
 // distinct key in the warp).
 __global__ void __launch_bounds__(GROUP_THREADS) k_group_count(const __grid_constant__ PlanDev P, uint32_t n,
-                                                               unsigned *count, uint16_t *keys) {
+                                                               uint32_t per_block, unsigned *count,
+                                                               uint16_t *keys) {
     __shared__ unsigned local[GPUMCD_MAX_SPECTRUM_BINS];
     const int nb = group_bins(P);
     const unsigned lt = lanemask_lt();
     // the block's histories in rounds of one per thread: the same trip count
     // for every thread, so whole warps take part in each match
-    const uint32_t j0 = blockIdx.x * GROUP_PER_BLOCK, jend = min(n, j0 + GROUP_PER_BLOCK);
+    const uint32_t j0 = blockIdx.x * per_block, jend = min(n, j0 + per_block);
     for (int i = threadIdx.x; i < nb; i += blockDim.x) local[i] = 0u;
     __syncthreads();
     for (uint32_t jb = j0; jb < jend; jb += blockDim.x) {
@@ -1426,14 +1432,14 @@ __global__ void __launch_bounds__(GROUP_SCAN_THREADS) k_group_scan(unsigned *cou
 // writes their offsets there (the order within a bin is not fixed: claims in
 // any order give the same tally).  The keys come from k_group_count.
 __global__ void __launch_bounds__(GROUP_THREADS) k_group_scatter(const __grid_constant__ PlanDev P, uint32_t n,
-                                                                 unsigned *cursor, const uint16_t *keys,
-                                                                 uint32_t *order) {
+                                                                 uint32_t per_block, unsigned *cursor,
+                                                                 const uint16_t *keys, uint32_t *order) {
     __shared__ unsigned local[GPUMCD_MAX_SPECTRUM_BINS];
     __shared__ unsigned base[GPUMCD_MAX_SPECTRUM_BINS];
     const int nb = group_bins(P);
     const int lane = threadIdx.x & 31;
     const unsigned lt = lanemask_lt();
-    const uint32_t j0 = blockIdx.x * GROUP_PER_BLOCK, jend = min(n, j0 + GROUP_PER_BLOCK);
+    const uint32_t j0 = blockIdx.x * per_block, jend = min(n, j0 + per_block);
     for (int i = threadIdx.x; i < nb; i += blockDim.x) local[i] = 0u;
     __syncthreads();
     for (uint32_t jb = j0; jb < jend; jb += blockDim.x) {
@@ -1466,10 +1472,11 @@ cudaError_t launch_group_order(const PlanDev &P, uint32_t n, unsigned *count, ui
     if (nb < 1 || nb > GPUMCD_MAX_SPECTRUM_BINS || n == 0 || !P.spec) return cudaErrorInvalidValue;
     cudaError_t e = cudaMemsetAsync(count, 0, (size_t)nb * sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
-    const unsigned blocks = (n + GROUP_PER_BLOCK - 1) / GROUP_PER_BLOCK;
-    k_group_count<<<blocks, GROUP_THREADS, 0, s>>>(P, n, count, keys);
+    const uint32_t per_block = group_per_block(n);
+    const unsigned blocks = (n + per_block - 1) / per_block;
+    k_group_count<<<blocks, GROUP_THREADS, 0, s>>>(P, n, per_block, count, keys);
     k_group_scan<<<1, GROUP_SCAN_THREADS, 0, s>>>(count, nb);
-    k_group_scatter<<<blocks, GROUP_THREADS, 0, s>>>(P, n, count, keys, order);
+    k_group_scatter<<<blocks, GROUP_THREADS, 0, s>>>(P, n, per_block, count, keys, order);
     return cudaGetLastError();
 }
 
