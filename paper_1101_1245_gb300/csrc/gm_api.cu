@@ -46,7 +46,7 @@ struct Plan {
     bool failed = false;     // a sequence failed: the tally is incomplete until plan_reset
     cudaEvent_t reset_done = nullptr;  // after the last plan_reset's memsets (any stream)
     DevBuf tally;   // [W][nvox] u64, then the ledger [4] u64
-    DevBuf spec;    // [2(n_spec+1)] floats
+    DevBuf spec;    // the spectrum (spec_words), or the phase-space records
     gpumcd_run_stats acc;  // counters accumulated over the plan's runs
 };
 
@@ -563,7 +563,7 @@ gpumcd_status gpumcd_plan_open(gpumcd_ctx *c, int32_t phantom_id, const gpumcd_s
     gpumcd_status st = dev_alloc(c, p.tally, ((size_t)n_batches * nvox + 4) * 8);
     DevBuf tmp;
     if (st == GPUMCD_OK && p.n_spec > 0) {
-        st = dev_alloc(c, p.spec, (size_t)2 * (p.n_spec + 1) * 4);
+        st = dev_alloc(c, p.spec, (size_t)spec_words(p.n_spec) * 4);
         if (st == GPUMCD_OK) st = dev_alloc(c, tmp, (size_t)(2 * p.n_spec + 1) * 8);
         if (st == GPUMCD_OK) {
             double *d = (double *)tmp.p;
@@ -1462,7 +1462,7 @@ gpumcd_status gpumcd_debug_sample(gpumcd_ctx *c, int32_t kind, double p0, int32_
     int ns = 0;
     if (st == GPUMCD_OK && kind == 5) {
         ns = src->n_spectrum;
-        st = dev_alloc(c, spec, (size_t)2 * (ns + 1) * 4);
+        st = dev_alloc(c, spec, (size_t)spec_words(ns) * 4);
         if (st == GPUMCD_OK) st = dev_alloc(c, tmp, (size_t)(2 * ns + 1) * 8);
         if (st == GPUMCD_OK) {
             double *d = (double *)tmp.p;

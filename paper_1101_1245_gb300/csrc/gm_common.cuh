@@ -53,6 +53,12 @@ __host__ __device__ constexpr int tab_el(int m) { return TAB_MAT + m * TAB_MAT_F
 __host__ __device__ constexpr uint32_t tab_bytes(int n) { return 4u * (uint32_t)(TAB_MAT + n * TAB_MAT_FLOATS); }
 static_assert(tab_bytes(1) % 16 == 0 && (4 * TAB_MAT_FLOATS) % 16 == 0, "bulk copies move multiples of 16 bytes");
 
+// A spectrum on the device: the CDF [n+1], the bin edges [n+1], then a guide of
+// SPEC_GUIDE words that bounds the search for a quantile z in ((j)/SPEC_GUIDE,
+// (j+1)/SPEC_GUIDE]: the first and last bin it can fall in (low, high half).
+constexpr int SPEC_GUIDE = 256;
+__host__ __device__ constexpr int spec_words(int n) { return 2 * (n + 1) + SPEC_GUIDE; }
+
 constexpr int MAJ_FLOATS = 2 * G;  // per phantom: photon majorant | electron majorant
 
 // Grid geometry: a table index is x = (ln E - ln E0) / d, evaluated as
@@ -100,7 +106,7 @@ struct __align__(16) PlanDev {
     unsigned long long *tally;     // [n_batches][nvox] energy in quanta
     unsigned long long *ledger;    // [incident, escaped, rest, spare]
     const float *maj;              // [photon G | electron G] majorants, 1/cm
-    const float *spec;             // spectrum: [n_spec+1 cdf | n_spec+1 edges], or null
+    const float *spec;             // spectrum (spec_words), or null
     int32_t nx, ny, nz, n_spec;
     float dx, dy, dz, inv_dx;
     float inv_dy, inv_dz, X, Y;

@@ -300,19 +300,40 @@ __global__ void k_majorants(const float *tab, const unsigned int *rho_max_bits, 
 }
 
 // Spectrum: FP64 prefix sum of the weights into a normalised CDF (the
-// inverse-CDF table), stored with the bin edges as floats.
+// inverse-CDF table), stored with the bin edges as floats and the guide of the
+// search in it (one warp: the sum on lane 0, then the guide).
 __global__ void k_spectrum(const double *edges, const double *w, int n, float *out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double tot = 0.0;
-    for (int i = 0; i < n; ++i) tot += w[i];
-    double acc = 0.0;
-    out[0] = 0.f;
-    for (int i = 0; i < n; ++i) {
-        acc += w[i];
-        out[i + 1] = (float)(acc / tot);
+    if (blockIdx.x != 0) return;
+    if (threadIdx.x == 0) {
+        double tot = 0.0;
+        for (int i = 0; i < n; ++i) tot += w[i];
+        double acc = 0.0;
+        out[0] = 0.f;
+        for (int i = 0; i < n; ++i) {
+            acc += w[i];
+            out[i + 1] = (float)(acc / tot);
+        }
+        out[n] = 1.f;
+        for (int i = 0; i <= n; ++i) out[n + 1 + i] = (float)edges[i];
     }
-    out[n] = 1.f;
-    for (int i = 0; i <= n; ++i) out[n + 1 + i] = (float)edges[i];
+    __syncwarp();
+    uint32_t *guide = reinterpret_cast<uint32_t *>(out) + 2 * (n + 1);
+    for (int j = threadIdx.x; j < SPEC_GUIDE; j += 32) {
+        // quantiles above y0 and up to y1: the first bin whose end is above y0
+        // to the first whose end reaches y1
+        const float y0 = (float)j / (float)SPEC_GUIDE, y1 = (float)(j + 1) / (float)SPEC_GUIDE;
+        int lo = 0, hi = n - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (out[mid + 1] > y0) hi = mid; else lo = mid + 1;
+        }
+        int lo1 = lo, hi1 = n - 1;
+        while (lo1 < hi1) {
+            const int mid = (lo1 + hi1) >> 1;
+            if (out[mid + 1] >= y1) hi1 = mid; else lo1 = mid + 1;
+        }
+        guide[j] = (uint32_t)lo | ((uint32_t)lo1 << 16);
+    }
 }
 
 // Fold of a plan's batch tallies (GPUMCD §II.D): mean dose per history and
