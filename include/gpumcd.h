@@ -244,7 +244,8 @@ gpumcd_status gpumcd_simulate_device(gpumcd_ctx *ctx, int32_t phantom_id,
  * (power of two in [8, 64]; 0 = 32) batch copies kept on the device.  The
  * plan's histories are numbered from 0 and its tally accumulates over runs, so
  * the result after N histories does not depend on how the runs were split or
- * on what other plans shared them. */
+ * on what other plans shared them.  The tally is zeroed on the context's
+ * stream; later calls on the plan come after that, on any stream. */
 gpumcd_status gpumcd_plan_open(gpumcd_ctx *ctx, int32_t phantom_id, const gpumcd_source *source,
                                uint64_t seed, uint32_t n_batches, int32_t *plan_id);
 

@@ -660,8 +660,22 @@ gpumcd_status gpumcd_plan_reset(gpumcd_ctx *c, int32_t plan_id, uint64_t seed, v
     ST(set_device(c));
     cudaStream_t s = pick(c, stream);
     Plan &p = it->second;
-    CK(cudaStreamWaitEvent(s, p.reset_done, 0));
-    CK(zero_tally(p, c->phantoms.at(p.phantom).nvox, s));
+    const uint64_t nvox = c->phantoms.at(p.phantom).nvox;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    CK(cudaStreamIsCapturing(s, &capture));
+    if (capture == cudaStreamCaptureStatusNone) {
+        CK(cudaStreamWaitEvent(s, p.reset_done, 0));
+        CK(zero_tally(p, nvox, s));
+    } else {
+        // a captured reset is a node of the caller's graph: it cannot wait for
+        // an event from outside, so the host does, and it records none
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        const cudaError_t e = cudaEventSynchronize(p.reset_done);
+        CK(cudaThreadExchangeStreamCaptureMode(&mode));
+        CK(e);
+        CK(cudaMemsetAsync(p.tally.p, 0, ((size_t)p.W * nvox + 4) * 8, s));
+    }
     p.seed = seed;
     p.hist_sub = 0;
     p.hist_done = 0;

@@ -38,3 +38,31 @@ def test_first_use_on_another_stream(how, n_batches):
         ctx.plan_close(plan)
     ctx.close()
     assert np.array_equal(doses[0], doses[1]) and np.array_equal(doses[0], doses[2])
+
+
+def test_reset_in_a_captured_graph():
+    """A reset may be captured: its replay zeroes the tally, and the plan stays usable."""
+    import torch
+    ph = W.homogeneous((16, 16, 16), 0.5, W.MAT_WATER, 1.0)
+    src = W.pencil(W.ELECTRON, 6.0, 4.0, 4.0)
+    ctx = make_ctx()
+    pid = ctx.create_phantom(ph)
+    plan = ctx.plan_open(pid, src, 11, 8)
+    d = torch.zeros(ph.nvox, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    doses = []
+    ctx.run([plan], [640])
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.plan_reset(plan, 11, torch.cuda.current_stream().cuda_stream)
+    for _ in range(2):
+        graph.replay()
+        torch.cuda.synchronize()
+        ctx.run([plan], [640])
+        st = ctx.plan_result(plan, 0.5, d.data_ptr())
+        assert st["e_incident"] == 640 * 6 << 26 and ledger_exact(st)
+        doses.append(d.cpu().numpy())
+        ctx.plan_reset(plan, 11)
+    ctx.plan_close(plan)
+    ctx.close()
+    assert np.array_equal(doses[0], doses[1])
