@@ -400,7 +400,7 @@ def run_c2(args):
     d2h = 4 * nvox * 8
 
     st_e, st_g = stats[-1]
-    launches = st_e["n_launches"] + st_g["n_launches"] + 2 * 3  # transport + fold, s_thr, ledger sum
+    launches = st_e["n_launches"] + st_g["n_launches"] + 2 * 2  # transport + fold, s_thr
     clocks = clk.summary()
     ev_e = st_e["n_electron_steps"] + st_e["n_photon_events"]
     ev_g = st_g["n_electron_steps"] + st_g["n_photon_events"]
@@ -661,7 +661,7 @@ def run_c4(args):
     # per round unless a queue overflowed): its folds
     folds = sum(x["n_launches"] for x in st)
     transport_launches = last["sequences"]
-    launches = transport_launches + 3 * folds  # + the fold and two s_thr kernels of every fold
+    launches = transport_launches + 2 * folds  # + the fold and the s_thr kernel of every fold
 
     # the plain form: the same plans one at a time, same seeds and schedule
     plain_runs = [timed(plain, i) for i in range(min(2, args.steps))]

@@ -80,7 +80,7 @@ struct Phys {
 enum { T_PH = 0, T_EL = 1, NT = 2 };
 
 // A particle record: 48 bytes, three 16-byte words.
-//   a = (x, y, z, ux), b = (uy, uz, E bits, history bits), c = (lineage lo, lineage hi, draw, plan)
+//   a = (x, y, z, ux), b = (uy, uz, E bits, history bits), c = (lineage a, lineage c (PhiloxLineage), draw, plan)
 struct __align__(16) Rec {
     float4 a;
     float4 b;

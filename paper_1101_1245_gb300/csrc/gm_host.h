@@ -33,8 +33,6 @@ int sthr_blocks(uint64_t nvox, int n_sm);
 // red: [D_max bits (in) | sum sigma/D | count | deposited | 0 (in) | ledger (4)]
 cudaError_t launch_sthr(const double *dose, const double *sigma, uint64_t nvox, double thr, void *part,
                         unsigned long long *red, const unsigned long long *ledger, int n_sm, cudaStream_t s);
-cudaError_t launch_sum_u64(const unsigned long long *a, uint64_t n, unsigned long long *out, int n_sm,
-                           cudaStream_t s);
 cudaError_t launch_fold_noalloc(int device, const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
                                 int W, uint64_t n_hist, double inv_vol, double thr, double *dose, double *sigma,
                                 cudaStream_t s, unsigned long long result[4]);

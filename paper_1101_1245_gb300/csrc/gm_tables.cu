@@ -680,16 +680,6 @@ __global__ void __launch_bounds__(kSthrThreads) k_sthr(const double *dose, const
     if (threadIdx.x < 4) red[5 + threadIdx.x] = ledger[threadIdx.x];
 }
 
-// Exact integer sum of a tally (for the energy ledger).
-__global__ void k_sum_u64(const unsigned long long *a, uint64_t n, unsigned long long *out) {
-    unsigned long long s = 0;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
-         i += (uint64_t)gridDim.x * blockDim.x)
-        s += a[i];
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0 && s) atomicAdd(out, s);
-}
-
 __global__ void k_philox(const uint4 *ctr, uint2 key, uint64_t n, uint4 *out) {
     const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     if (i < n) out[i] = philox4x32_10(ctr[i], key);
@@ -814,14 +804,6 @@ int sthr_blocks(uint64_t nvox, int n_sm) {
 cudaError_t launch_sthr(const double *dose, const double *sigma, uint64_t nvox, double thr, void *part,
                         unsigned long long *red, const unsigned long long *ledger, int n_sm, cudaStream_t s) {
     k_sthr<<<sthr_blocks(nvox, n_sm), kSthrThreads, 0, s>>>(dose, sigma, nvox, thr, (double2 *)part, red, ledger);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sum_u64(const unsigned long long *a, uint64_t n, unsigned long long *out, int n_sm,
-                           cudaStream_t s) {
-    uint64_t blocks = (n + 255) / 256;
-    const uint64_t cap = (uint64_t)n_sm * 8;
-    k_sum_u64<<<(int)(blocks < cap ? (blocks ? blocks : 1) : cap), 256, 0, s>>>(a, n, out);
     return cudaGetLastError();
 }
 

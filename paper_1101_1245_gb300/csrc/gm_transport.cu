@@ -2,8 +2,9 @@
 //
 // One launch runs every particle it can reach to completion.  Each warp holds
 // 32 particles of ONE type (photon or electron) in registers and advances all
-// of them by one event per iteration: a Woodcock flight for photons (GPUMCD
-// §II.A) or one condensed-history step for electrons (§II.B.3).  Lanes whose
+// of them together: up to four Woodcock flights and the real event they end on
+// for photons (GPUMCD §II.A), up to four condensed-history steps for electrons
+// (§II.B.3).  Lanes whose
 // particle ended are refilled, in this order, from the warp's private stack of
 // that type, from the global overflow queue of the previous launch, and from
 // the primaries of the launch's plans (claimed in chunks).  Secondaries go to
