@@ -301,39 +301,48 @@ __global__ void k_majorants(const float *tab, const unsigned int *rho_max_bits, 
 
 // Spectrum: FP64 prefix sum of the weights into a normalised CDF (the
 // inverse-CDF table), stored with the bin edges as floats and the guide of the
-// search in it (one warp: the sum on lane 0, then the guide).
-__global__ void k_spectrum(const double *edges, const double *w, int n, float *out) {
-    if (blockIdx.x != 0) return;
+// search in it.  One block: the sum runs on one thread, in the bins' order,
+// over shared memory; the divisions and the guide's searches on all.  Opening
+// a plan of 256 bins takes 52 us with it, 178 with one thread that summed,
+// divided and copied from global memory (1024 bins: 96, 549).
+constexpr int kSpectrumThreads = SPEC_GUIDE;
+
+__global__ void __launch_bounds__(kSpectrumThreads) k_spectrum(const double *edges, const double *w, int n,
+                                                               float *out) {
+    __shared__ double acc[GPUMCD_MAX_SPECTRUM_BINS];
+    __shared__ float cdf[GPUMCD_MAX_SPECTRUM_BINS + 1];
+    for (int i = threadIdx.x; i < n; i += kSpectrumThreads) acc[i] = w[i];
+    __syncthreads();
     if (threadIdx.x == 0) {
-        double tot = 0.0;
-        for (int i = 0; i < n; ++i) tot += w[i];
-        double acc = 0.0;
-        out[0] = 0.f;
+        double a = 0.0;
         for (int i = 0; i < n; ++i) {
-            acc += w[i];
-            out[i + 1] = (float)(acc / tot);
+            a += acc[i];
+            acc[i] = a;
         }
-        out[n] = 1.f;
-        for (int i = 0; i <= n; ++i) out[n + 1 + i] = (float)edges[i];
     }
-    __syncwarp();
-    uint32_t *guide = reinterpret_cast<uint32_t *>(out) + 2 * (n + 1);
-    for (int j = threadIdx.x; j < SPEC_GUIDE; j += 32) {
-        // quantiles above y0 and up to y1: the first bin whose end is above y0
-        // to the first whose end reaches y1
-        const float y0 = (float)j / (float)SPEC_GUIDE, y1 = (float)(j + 1) / (float)SPEC_GUIDE;
-        int lo = 0, hi = n - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (out[mid + 1] > y0) hi = mid; else lo = mid + 1;
-        }
-        int lo1 = lo, hi1 = n - 1;
-        while (lo1 < hi1) {
-            const int mid = (lo1 + hi1) >> 1;
-            if (out[mid + 1] >= y1) hi1 = mid; else lo1 = mid + 1;
-        }
-        guide[j] = (uint32_t)lo | ((uint32_t)lo1 << 16);
+    __syncthreads();
+    const double tot = acc[n - 1];
+    for (int i = threadIdx.x; i <= n; i += kSpectrumThreads) {
+        cdf[i] = i == 0 ? 0.f : i == n ? 1.f : (float)(acc[i - 1] / tot);
+        out[i] = cdf[i];
+        out[n + 1 + i] = (float)edges[i];
     }
+    __syncthreads();
+    // quantiles above y0 and up to y1: the first bin whose end is above y0 to
+    // the first whose end reaches y1
+    const int j = threadIdx.x;
+    const float y0 = (float)j / (float)SPEC_GUIDE, y1 = (float)(j + 1) / (float)SPEC_GUIDE;
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (cdf[mid + 1] > y0) hi = mid; else lo = mid + 1;
+    }
+    int lo1 = lo, hi1 = n - 1;
+    while (lo1 < hi1) {
+        const int mid = (lo1 + hi1) >> 1;
+        if (cdf[mid + 1] >= y1) hi1 = mid; else lo1 = mid + 1;
+    }
+    reinterpret_cast<uint32_t *>(out)[2 * (n + 1) + j] = (uint32_t)lo | ((uint32_t)lo1 << 16);
 }
 
 // Fold of a plan's batch tallies (GPUMCD §II.D): mean dose per history and
@@ -749,7 +758,7 @@ cudaError_t launch_majorants(const float *tab, const unsigned int *rho_max_bits,
 }
 
 cudaError_t launch_spectrum(const double *edges, const double *w, int n, float *out, cudaStream_t s) {
-    k_spectrum<<<1, 32, 0, s>>>(edges, w, n, out);
+    k_spectrum<<<1, kSpectrumThreads, 0, s>>>(edges, w, n, out);
     return cudaGetLastError();
 }
 
