@@ -371,7 +371,10 @@ struct FoldConst {
     double k_sigma;  // ... times sqrt(W / (W - 1)) (unequal batches) or sqrt(1 / (W - 1)) (equal)
     double inv_n;    // 1 / N
     double q_n;      // (N div W) / N
+    double n_tot;    // N
+    double n_each;   // N div W
     double n1, n0;   // r and W - r
+    float m1, m0;    // the same
     uint32_t r;      // N mod W: the batches with one history more
 };
 
@@ -468,17 +471,29 @@ __device__ __forceinline__ double sqrt_fold(double v) {
     return __hiloint2double(__double2hiint(s) + (((ex - odd) >> 1) << 20), __double2loint(s));
 }
 
-// The two-pass form in FP64, for sums of squares beyond 128 bits (far beyond
-// realistic tallies): sum_b (S_b - n_b D)^2.
+// The two-pass form in FP64, sum_b (S_b - n_b D)^2, for sums of squares beyond
+// 128 bits (far beyond realistic tallies) and for unequal batches too tight for
+// the moments below.  Each difference is rounded once, and the rounding of the
+// mean is common to them: as sum_b (S_b - n_b D) = 0, it leaves the result alone
+// to first order but for the one history more of the first r batches.  (Means
+// of n_b histories formed as products, (N div W) D and that plus D, are rounded
+// apart: with 100 histories a batch that scatter by 1e-6 the result is off by
+// 5e-10 that way, by 4e-12 this way.)
 __device__ __noinline__ double two_pass(const unsigned long long *tally, uint64_t nvox, int W, uint64_t v, double tot,
                                         const FoldConst &fc) {
-    const double a0 = tot * fc.q_n, a1 = fma(tot, fc.inv_n, a0);
+    const double mean = tot / fc.n_tot, each = tot * fc.q_n;  // each: exact for equal batches, q_n = 1 / W
     double acc = 0.0;
     for (int b = 0; b < W; ++b) {
-        const double t = (double)tally[(uint64_t)b * nvox + v] - (b < (int)fc.r ? a1 : a0);
+        const double s = (double)tally[(uint64_t)b * nvox + v];
+        const double t = fc.r == 0 ? s - each : fma(-(fc.n_each + (b < (int)fc.r ? 1.0 : 0.0)), mean, s);
         acc = fma(t, t, acc);
     }
     return acc;
+}
+
+// |x| toward zero as a float of 20 fraction bits, by integer instructions (0 below 2^-127).
+__device__ __forceinline__ float top_float(double x) {
+    return __int_as_float(max((__double2hiint(x) & 0x7FFFFFFF) - 0x38000000, 0) << 3);
 }
 
 // Equal batches (n_b = N / W for every b): the variance numerator is formed
@@ -520,8 +535,16 @@ __device__ __forceinline__ void fold_voxel_equal(const unsigned long long *tally
 // u_b = S_b - i, S_b - n_b D = u_b - f, where f is f0, plus D for the first r
 // batches; so, with U1 and U0 the sums of u_b over these and over the others,
 //   sum_b (S_b - n_b D)^2 = sum u_b^2 + f1 (r f1 - 2 U1) + f0 ((W-r) f0 - 2 U0).
-// The sums of u_b follow exactly, in 128-bit integers, from those of S_b, and,
-// the u_b being centred, the terms are of the result's own size.
+// The sums of u_b follow exactly, in 128-bit integers, from those of S_b.  With
+// F = r f1^2 + (W-r) f0^2 the terms are at most nine times the larger of the
+// result and F, so they lose nothing while the result is not below F: while the
+// batches scatter by the mean energy of a history or more.  Every voxel of a
+// tally in earnest does (a history's deposit there varies by its own size);
+// where a few histories deposit nearly the same energy, as in one coarse voxel
+// that absorbs them all, the two-pass form takes over.  (With 100 histories a
+// batch the moments alone are off by 4e-14 of the variance where a history's
+// deposit scatters by 1%, by 2e-6 where it does by 1e-6, and not zero where it
+// does not at all.  The test costs 256^3 voxels up to 1% of a result call.)
 template <int W>
 __device__ __forceinline__ void fold_voxel(const unsigned long long *tally, const uint32_t *vox, uint64_t nvox,
                                            uint64_t v, const FoldConst &fc, double &dv, double &sv,
@@ -543,8 +566,9 @@ __device__ __forceinline__ void fold_voxel(const unsigned long long *tally, cons
     dv = sv = 0.0;
     if (tot == 0ull) return;
     const double td = u128_to_double(U128{tot, 0ull});
-    double acc;
-    if (sq.hi < (1ull << 57)) {
+    double acc = 0.0;
+    bool moments = sq.hi < (1ull << 57);
+    if (moments) {
         const double a0 = td * fc.q_n;
         // i and f0 from a0's bits (its exponent is below 63: a0 < S / W)
         const int ex = (__double2hiint(a0) >> 20) - 1023;
@@ -576,9 +600,11 @@ __device__ __forceinline__ void fold_voxel(const unsigned long long *tally, cons
         acc = u128_to_double(q);
         acc = fma(f1, fma(fc.n1, f1, scaled((unsigned long long)(u1 < 0 ? -u1 : u1), 1, u1 > 0)), acc);
         acc = fma(f0, fma(fc.n0, f0, scaled((unsigned long long)(u0 < 0 ? -u0 : u0), 1, u0 > 0)), acc);
-    } else {
-        acc = two_pass(tally, nvox, W, v, td, fc);
+        const float g1 = top_float(f1), g0 = top_float(f0);
+        const float F = fmaf(fc.m1 * g1, g1, fc.m0 * g0 * g0);
+        moments = !(top_float(acc) < F);
     }
+    if (!moments) acc = two_pass(tally, nvox, W, v, td, fc);
     const double y = rcp_code(code);
     dv = td * fc.k_dose * y;
     sv = sqrt_fold(acc) * fc.k_sigma * y;
@@ -769,6 +795,10 @@ static FoldConst fold_const(int W, uint64_t n_hist, double inv_vol) {
     fc.r = (uint32_t)(n_hist % (uint64_t)W);
     fc.n1 = (double)fc.r;
     fc.n0 = (double)(W - (int)fc.r);
+    fc.m1 = (float)fc.n1;
+    fc.m0 = (float)fc.n0;
+    fc.n_tot = (double)n_hist;
+    fc.n_each = (double)(n_hist / (uint64_t)W);
     fc.inv_n = (double)(1.0L / N);
     fc.q_n = (double)((long double)(n_hist / (uint64_t)W) / N);
     const long double k = (long double)kQ * kMeVPerGramToGy * inv_vol * (1.0L / (long double)kRhoQ) / N;
