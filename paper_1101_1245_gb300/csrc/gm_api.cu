@@ -1019,6 +1019,11 @@ gpumcd_status seq_finish(gpumcd_ctx *c, Slot &sl) {
         result = launch_one(c, sl);
         if (result != GPUMCD_OK) break;
     }
+    if (result != GPUMCD_OK) {
+        // a launch may have been enqueued before the call that failed: nothing
+        // is pending on the slot's buffers and the plans' tallies when they are free
+        if (cudaStreamSynchronize(sl.s) != cudaSuccess) cudaGetLastError();
+    }
     float ms = 0.f;  // from the first launch's start to the last one's end
     if (cudaEventElapsedTime(&ms, sl.ev0, sl.ev1) != cudaSuccess) {
         cudaGetLastError();
