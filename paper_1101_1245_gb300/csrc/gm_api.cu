@@ -735,9 +735,10 @@ void first_queues(gpumcd_ctx *c, Slot &sl) {
 
 // First launch of a sequence from the slot's captured graph.  Its copy nodes
 // touch only slot-owned buffers of fixed size (the whole plan table is
-// copied), so the graph stays valid for the slot's lifetime and
-// only the kernel node's argument block changes between runs; a new launch
-// shape (grid, CTA size, kernel variant) is captured afresh.
+// copied), so the graph stays valid for the slot's lifetime and only the
+// kernel node's argument block and shared memory (the loaded materials'
+// tables) change between runs; a new launch shape (grid, CTA size, kernel
+// variant) is captured afresh.
 gpumcd_status first_launch_graph(gpumcd_ctx *c, Slot &sl) {
     first_queues(c, sl);
     Control *dc = &((SeqStart *)sl.start.p)->control;
@@ -784,6 +785,7 @@ gpumcd_status first_launch_graph(gpumcd_ctx *c, Slot &sl) {
         void *args[] = {&sl.A};
         kp.kernelParams = args;
         kp.extra = nullptr;
+        kp.sharedMemBytes = (unsigned)transport_smem_bytes(sl.A.tab_bytes);  // the loaded materials may be others
         CK(cudaGraphExecKernelNodeSetParams(sl.gexec, sl.knode, &kp));
     }
     CK(cudaEventRecord(sl.ev0, sl.s));

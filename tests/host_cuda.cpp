@@ -28,6 +28,7 @@ struct Node {
     const void *src;
     size_t n;
     const void *fn;
+    unsigned shared;  // bytes of dynamic shared memory
     gm::TransportArgs args;
 };
 struct Graph {
@@ -41,6 +42,7 @@ struct Exec {
 std::map<std::string, long> calls;
 std::map<std::string, long> fail_at;
 int leave = 0;
+long misfits = 0;
 std::vector<Stream *> streams;
 std::vector<const void *> launched;  // compiled kernels, by launch
 
@@ -54,8 +56,9 @@ bool fails(const char *name) {
 
 Stream *of(cudaStream_t s) { return (Stream *)s; }
 
-void kernel(const gm::TransportArgs &a, const void *fn, Stream *s) {
+void kernel(const gm::TransportArgs &a, const void *fn, unsigned shared, Stream *s) {
     ++s->issued;
+    if (shared != gm::transport_smem_bytes(a.tab_bytes)) ++misfits;
     launched.push_back(fn);
     if (leave > 0) {
         --leave;
@@ -73,6 +76,7 @@ void host_cuda_reset() {
     fail_at.clear();
     launched.clear();
     leave = 0;
+    misfits = 0;
 }
 void host_cuda_leave(int launches) { leave = launches; }
 void host_cuda_fail(const char *name, int nth_from_now) { fail_at[name] = calls[name] + nth_from_now; }
@@ -82,6 +86,8 @@ long host_cuda_pending() {
     for (Stream *s : streams) n += s->issued - s->done;
     return n;
 }
+// launches whose shared memory is not the size their tables take
+long host_cuda_misfits() { return misfits; }
 long host_cuda_launched(const void **fn, long max) {
     for (long i = 0; i < max && i < (long)launched.size(); ++i) fn[i] = launched[i];
     return (long)launched.size();
@@ -146,7 +152,7 @@ cudaError_t cudaMemsetAsync(void *p, int v, size_t n, cudaStream_t) {
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t st) {
     CALL(cudaMemcpyAsync);
     if (of(st)->capture)
-        of(st)->capture->nodes.push_back(new Node{0, d, s, n, nullptr, {}});
+        of(st)->capture->nodes.push_back(new Node{0, d, s, n, nullptr, 0, {}});
     else
         memcpy(d, s, n);
     return cudaSuccess;
@@ -187,6 +193,7 @@ cudaError_t cudaGraphNodeGetType(cudaGraphNode_t n, cudaGraphNodeType *t) {
 cudaError_t cudaGraphKernelNodeGetParams(cudaGraphNode_t n, cudaKernelNodeParams *p) {
     memset(p, 0, sizeof *p);
     p->func = const_cast<void *>(((Node *)n)->fn);
+    p->sharedMemBytes = ((Node *)n)->shared;
     return cudaSuccess;
 }
 cudaError_t cudaGraphExecKernelNodeSetParams(cudaGraphExec_t x, cudaGraphNode_t n, const cudaKernelNodeParams *p) {
@@ -195,6 +202,7 @@ cudaError_t cudaGraphExecKernelNodeSetParams(cudaGraphExec_t x, cudaGraphNode_t 
     for (size_t i = 0; i < e.nodes.size(); ++i)
         if (e.of[i] == (const Node *)n) {
             e.nodes[i].fn = p->func;
+            e.nodes[i].shared = p->sharedMemBytes;
             e.nodes[i].args = *(const gm::TransportArgs *)p->kernelParams[0];
             return cudaSuccess;
         }
@@ -204,7 +212,7 @@ cudaError_t cudaGraphLaunch(cudaGraphExec_t x, cudaStream_t s) {
     CALL(cudaGraphLaunch);
     for (const Node &n : ((Exec *)x)->nodes) {
         if (n.kind)
-            kernel(n.args, n.fn, of(s));
+            kernel(n.args, n.fn, n.shared, of(s));
         else
             memcpy(n.dst, n.src, n.n);
     }
@@ -249,6 +257,7 @@ cudaError_t launch_group_order(const PlanDev &, uint32_t, unsigned *, uint16_t *
 }
 cudaError_t launch_debug_sample(const float *, const Phys &, int, float, int, const float *, int, uint64_t, uint64_t,
                                 float *, cudaStream_t) { return cudaSuccess; }
+size_t transport_smem_bytes(uint32_t tab_bytes) { return 16384 + tab_bytes; }
 cudaError_t transport_configure() { return cudaSuccess; }
 // one compiled kernel for each combination of the two, as far as host code can tell
 const void *transport_kernel(const TransportArgs &a, int, int) {
@@ -258,10 +267,11 @@ const void *transport_kernel(const TransportArgs &a, int, int) {
 cudaError_t launch_transport(const TransportArgs &a, int grid, int block, int bps, cudaStream_t s) {
     if (fails("launch_transport")) return cudaErrorUnknown;
     const void *fn = transport_kernel(a, block, bps);
+    const unsigned shared = (unsigned)transport_smem_bytes(a.tab_bytes);
     if (of(s)->capture)
-        of(s)->capture->nodes.push_back(new Node{1, nullptr, nullptr, 0, fn, a});
+        of(s)->capture->nodes.push_back(new Node{1, nullptr, nullptr, 0, fn, shared, a});
     else
-        kernel(a, fn, of(s));
+        kernel(a, fn, shared, of(s));
     (void)grid;
     return cudaSuccess;
 }

@@ -22,7 +22,8 @@ def library() -> C.CDLL:
     for name, (res, args) in g.SIGNATURES.items():
         f = getattr(L, name)
         f.restype, f.argtypes = res, args
-    L.host_cuda_calls.restype = L.host_cuda_pending.restype = L.host_cuda_launched.restype = C.c_long
+    for f in (L.host_cuda_calls, L.host_cuda_pending, L.host_cuda_launched, L.host_cuda_misfits):
+        f.restype = C.c_long
     L.host_cuda_calls.argtypes = [C.c_char_p]
     L.host_cuda_fail.argtypes = [C.c_char_p, C.c_int]
     L.host_cuda_launched.argtypes = [C.c_void_p, C.c_long]
