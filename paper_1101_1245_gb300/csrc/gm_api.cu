@@ -66,6 +66,16 @@ struct SeqStart {
     PlanDev plans[GPUMCD_MAX_PLANS_PER_RUN];
 };
 
+// GPUMCD_LAUNCH_GRAPH: the first launch of a sequence (one upload of control
+// block and plan table, the kernel, the control read-back), captured and
+// replayed with the kernel's arguments updated.
+struct LaunchGraph {
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    cudaGraphNode_t kernel = nullptr;
+    int grid = 0, block = 0;
+};
+
 // Scratch and state of one launch sequence (the persistent kernel, then
 // relaunches over the overflow queues until they are empty).  Slot 0 serves
 // gpumcd_run on the caller's stream; slots 1..GPUMCD_MAX_INFLIGHT serve
@@ -86,14 +96,7 @@ struct Slot {
     unsigned long long in_count[NT] = {0, 0};
     std::vector<int32_t> ids;
     std::vector<uint64_t> n_hist;
-    // GPUMCD_LAUNCH_GRAPH: the first launch of a sequence (plan-table copy,
-    // control reset, kernel, control read-back) captured once per launch
-    // shape and replayed with the kernel's arguments updated
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t gexec = nullptr;
-    cudaGraphNode_t knode = nullptr;
-    int g_grid = 0, g_block = 0, g_bps = 0;
-    const void *g_fn = nullptr;  // the transport kernel the graph holds
+    std::map<const void *, LaunchGraph> graphs;  // by the transport kernel they hold
 };
 
 }  // namespace
@@ -273,6 +276,12 @@ gpumcd_status ensure_slot(gpumcd_ctx *c, Slot &sl, int grid, int block) {
     return GPUMCD_OK;
 }
 
+void free_graph(LaunchGraph &g) {
+    if (g.exec) cudaGraphExecDestroy(g.exec);
+    if (g.graph) cudaGraphDestroy(g.graph);
+    g = LaunchGraph{};
+}
+
 void free_slot(gpumcd_ctx *c, Slot &sl) {
     if (sl.busy && sl.s) cudaStreamSynchronize(sl.s);
     dev_free(c, sl.order);
@@ -286,8 +295,7 @@ void free_slot(gpumcd_ctx *c, Slot &sl) {
     if (sl.h_start) cudaFreeHost(sl.h_start);
     if (sl.ev0) cudaEventDestroy(sl.ev0);
     if (sl.ev1) cudaEventDestroy(sl.ev1);
-    if (sl.gexec) cudaGraphExecDestroy(sl.gexec);
-    if (sl.graph) cudaGraphDestroy(sl.graph);
+    for (auto &kv : sl.graphs) free_graph(kv.second);
     if (sl.own) cudaStreamDestroy(sl.own);
     sl = Slot{};
 }
@@ -733,63 +741,63 @@ void first_queues(gpumcd_ctx *c, Slot &sl) {
     }
 }
 
+// Capture the first launch of a slot's sequence.
+cudaError_t capture_graph(Slot &sl, LaunchGraph &g) {
+    Control *dc = &((SeqStart *)sl.start.p)->control;
+    cudaError_t e = cudaStreamBeginCapture(sl.s, cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    e = cudaMemcpyAsync(sl.start.p, sl.h_start, sizeof(SeqStart), cudaMemcpyHostToDevice, sl.s);
+    if (e == cudaSuccess) e = launch_transport(sl.A, sl.grid, sl.block, sl.bps, sl.s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(sl.h_control, dc, sizeof(Control), cudaMemcpyDeviceToHost, sl.s);
+    const cudaError_t e2 = cudaStreamEndCapture(sl.s, &g.graph);
+    if (e == cudaSuccess) e = e2;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&g.exec, g.graph, 0);
+    size_t n = 0;
+    if (e == cudaSuccess) e = cudaGraphGetNodes(g.graph, nullptr, &n);
+    std::vector<cudaGraphNode_t> nodes(n);
+    if (e == cudaSuccess) e = cudaGraphGetNodes(g.graph, nodes.data(), &n);
+    for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
+        cudaGraphNodeType ty;
+        e = cudaGraphNodeGetType(nodes[i], &ty);
+        if (e == cudaSuccess && ty == cudaGraphNodeTypeKernel) g.kernel = nodes[i];
+    }
+    if (e == cudaSuccess && !g.kernel) e = cudaErrorUnknown;
+    g.grid = sl.grid;
+    g.block = sl.block;
+    return e;
+}
+
 // First launch of a sequence from the slot's captured graph.  Its copy nodes
 // touch only slot-owned buffers of fixed size (the whole plan table is
 // copied), so the graph stays valid for the slot's lifetime and only the
 // kernel node's argument block and shared memory (the loaded materials'
-// tables) change between runs; a new launch shape (grid, CTA size, kernel
-// variant) is captured afresh.
+// tables) change between runs.  A kernel node keeps the function it was
+// captured with, so a slot keeps one graph for each compiled transport kernel
+// it has run (one plan or several, phase-space sources, photon-only mode ...),
+// captured again for another launch shape of that kernel.  With one graph a
+// slot, runs of one plan and of two in turn captured it at every call: 72 us
+// a call of 64 photons a plan, 54 with both kept (54 for direct launches too).
 gpumcd_status first_launch_graph(gpumcd_ctx *c, Slot &sl) {
     first_queues(c, sl);
-    Control *dc = &((SeqStart *)sl.start.p)->control;
-    // a graph is rebuilt for a new launch shape or another compiled kernel
-    // (its kernel node keeps the function it was captured with)
-    const void *fn = transport_kernel(sl.A, sl.block, sl.bps);
-    if (!sl.gexec || sl.g_grid != sl.grid || sl.g_block != sl.block || sl.g_bps != sl.bps || sl.g_fn != fn) {
-        if (sl.gexec) cudaGraphExecDestroy(sl.gexec);
-        if (sl.graph) cudaGraphDestroy(sl.graph);
-        sl.gexec = nullptr;
-        sl.graph = nullptr;
-        sl.knode = nullptr;
-        CK(cudaStreamBeginCapture(sl.s, cudaStreamCaptureModeThreadLocal));
-        cudaError_t e = cudaMemcpyAsync(sl.start.p, sl.h_start, sizeof(SeqStart), cudaMemcpyHostToDevice, sl.s);
-        if (e == cudaSuccess) e = launch_transport(sl.A, sl.grid, sl.block, sl.bps, sl.s);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(sl.h_control, dc, sizeof(Control), cudaMemcpyDeviceToHost, sl.s);
-        cudaGraph_t g = nullptr;
-        const cudaError_t e2 = cudaStreamEndCapture(sl.s, &g);
-        if (e == cudaSuccess) e = e2;
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&sl.gexec, g, 0);
+    LaunchGraph &g = sl.graphs[transport_kernel(sl.A, sl.block, sl.bps)];
+    if (!g.exec || g.grid != sl.grid || g.block != sl.block) {
+        free_graph(g);
+        const cudaError_t e = capture_graph(sl, g);
         if (e != cudaSuccess) {
-            if (g) cudaGraphDestroy(g);
-            sl.gexec = nullptr;
+            free_graph(g);
             return cuda_status(e);
         }
-        sl.graph = g;
-        size_t n = 0;
-        CK(cudaGraphGetNodes(g, nullptr, &n));
-        std::vector<cudaGraphNode_t> nodes(n);
-        CK(cudaGraphGetNodes(g, nodes.data(), &n));
-        for (cudaGraphNode_t nd : nodes) {
-            cudaGraphNodeType ty;
-            CK(cudaGraphNodeGetType(nd, &ty));
-            if (ty == cudaGraphNodeTypeKernel) sl.knode = nd;
-        }
-        if (!sl.knode) return GPUMCD_ERR_CUDA;
-        sl.g_grid = sl.grid;
-        sl.g_block = sl.block;
-        sl.g_bps = sl.bps;
-        sl.g_fn = fn;
     } else {
         cudaKernelNodeParams kp;
-        CK(cudaGraphKernelNodeGetParams(sl.knode, &kp));
+        CK(cudaGraphKernelNodeGetParams(g.kernel, &kp));
         void *args[] = {&sl.A};
         kp.kernelParams = args;
         kp.extra = nullptr;
         kp.sharedMemBytes = (unsigned)transport_smem_bytes(sl.A.tab_bytes);  // the loaded materials may be others
-        CK(cudaGraphExecKernelNodeSetParams(sl.gexec, sl.knode, &kp));
+        CK(cudaGraphExecKernelNodeSetParams(g.exec, g.kernel, &kp));
     }
     CK(cudaEventRecord(sl.ev0, sl.s));
-    CK(cudaGraphLaunch(sl.gexec, sl.s));
+    CK(cudaGraphLaunch(g.exec, sl.s));
     CK(cudaEventRecord(sl.ev1, sl.s));
     sl.k = 1;
     return GPUMCD_OK;

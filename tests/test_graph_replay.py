@@ -1,5 +1,7 @@
 """Replay of a sequence's first launch from a captured graph (GPUMCD_LAUNCH_GRAPH),
 with CUDA calls faked on the host: what each replay hands the kernel."""
+import ctypes as C
+
 import pytest
 
 import paper_1101_1245_gb300 as g
@@ -35,3 +37,46 @@ def test_shared_memory_follows_the_loaded_materials(ctx):
         ctx.destroy_phantom(pid)
     assert L.host_cuda_calls(b"cudaGraphLaunch") == 3
     assert L.host_cuda_misfits() == 0
+
+
+def test_alternating_kernels_are_captured_once(ctx):
+    """One plan and several run different compiled kernels: runs that alternate
+    rewrite arguments and capture nothing after each kernel's first run."""
+    L = library()
+    pid, a = open_plan(ctx)
+    _, b = open_plan(ctx)
+    for _ in range(5):
+        ctx.run([a], [100])
+        ctx.run([a, b], [100, 100])
+    assert L.host_cuda_calls(b"cudaGraphLaunch") == 10
+    assert L.host_cuda_calls(b"cudaGraphInstantiate") == 2
+    fn = (C.c_void_p * 10)()
+    assert L.host_cuda_launched(fn, 10) == 10
+    assert len({fn[i] for i in range(0, 10, 2)}) == len({fn[i] for i in range(1, 10, 2)}) == 1
+    assert fn[0] != fn[1]
+
+
+def test_another_launch_shape_is_captured_again(ctx):
+    L = library()
+    _, a = open_plan(ctx)
+    for threads in (1024, 512, 512, 1024):
+        ctx.set_launch(block_threads=threads, flags=g.LAUNCH_GRAPH)
+        ctx.run([a], [100])
+    assert L.host_cuda_calls(b"cudaGraphInstantiate") == 3
+    assert L.host_cuda_calls(b"cudaGraphExecDestroy") == 2
+
+
+@pytest.mark.parametrize("call", ["cudaStreamBeginCapture", "cudaGraphInstantiate", "cudaGraphGetNodes",
+                                  "cudaGraphExecKernelNodeSetParams", "cudaGraphLaunch"])
+def test_a_failed_capture_is_reported_and_tried_again(ctx, call):
+    L = library()
+    _, a = open_plan(ctx)
+    if call == "cudaGraphExecKernelNodeSetParams":
+        ctx.run([a], [100])
+    L.host_cuda_fail(call.encode(), 1)
+    with pytest.raises(g.GpumcdError) as e:
+        ctx.run([a], [100])
+    assert e.value.status == g.ERR_CUDA and L.host_cuda_pending() == 0
+    ctx.plan_reset(a, 1)
+    ctx.run([a], [100])
+    assert ctx.plan_histories(a) == 100
