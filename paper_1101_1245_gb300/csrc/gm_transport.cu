@@ -37,6 +37,9 @@ namespace gm {
 constexpr float kHardMajorantMargin = 1.00006103515625f;
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int MAX_WARPS = 32;
+// A warp's row of event counters: those before the cycle profile, then the hard passes.
+constexpr int CNT_ROW = CNT_PROF_CYC + 1;
+__host__ __device__ constexpr int row_word(int which) { return which == CNT_HARD_PASSES ? CNT_ROW - 1 : which; }
 
 struct WarpState {
     unsigned int stk[2];
@@ -58,7 +61,7 @@ struct Smem {
     const float *tab;
     PlanDev *plans;
     WarpState *ws;
-    unsigned int *wcnt;          // [MAX_WARPS][CNT_N] event counters, a row per warp
+    unsigned int *wcnt;          // [MAX_WARPS][CNT_ROW] event counters, a row per warp
     unsigned long long *cnt;     // [CNT_N] cycle profile (64-bit)
     unsigned int *ledger;        // [n_plans][3][2]: incident, escaped, rest; low and high words
 };
@@ -203,7 +206,7 @@ __device__ __forceinline__ void ledger_add(const Smem &S, uint32_t plan, int whi
 // photons) of transport, 2.38 and 5.33 before; the 2 MeV pencil of 1e5
 // photons 0.134 ms, 0.192 before.
 __device__ __forceinline__ unsigned int *counter(const Smem &S, int w, int which) {
-    return &S.wcnt[w * CNT_N + which];
+    return &S.wcnt[w * CNT_ROW + row_word(which)];
 }
 __device__ __forceinline__ void count(const Smem &S, int w, int which) { atomicAdd(counter(S, w, which), 1u); }
 
@@ -816,9 +819,14 @@ struct CtaFlags {
 // mbarrier and the source flags (fixed size, rounded up to 128 bytes), then the
 // tables staged by the bulk copy.
 constexpr size_t SMEM_FIXED = (sizeof(PlanDev) * GPUMCD_MAX_PLANS_PER_RUN + sizeof(WarpState) * MAX_WARPS +
-                               sizeof(unsigned int) * MAX_WARPS * CNT_N +
+                               sizeof(unsigned int) * MAX_WARPS * CNT_ROW +
                                sizeof(unsigned long long) * (CNT_N + 3 * GPUMCD_MAX_PLANS_PER_RUN + 1) +
                                sizeof(CtaFlags) + 127) / 128 * 128;
+// Three CTAs stay resident (block_threads <= 256 with blocks_per_sm = 3) with
+// every material loaded: an SM has 228 KB, of which each CTA takes 1 KB besides.
+// With counter rows of all CNT_N words only two did: 256 x 3 took 2.37 ms for 1e6
+// electrons of 15 MeV and 2.92 for 2e6 photons on 128^3 water, 2.10 and 2.54 so.
+static_assert(3 * (SMEM_FIXED + TAB_BYTES + 1024) <= 228 * 1024, "three CTAs of all materials");
 
 // Move the top n records of stack `t` to the global overflow queue.  A full
 // queue sets GPUMCD_ERR_QUEUE_OVERFLOW: the run is then invalid and reported,
@@ -1065,7 +1073,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
     PlanDev *plans = (PlanDev *)smem_raw;
     WarpState *ws = (WarpState *)(plans + GPUMCD_MAX_PLANS_PER_RUN);
     unsigned int *wcnt = (unsigned int *)(ws + MAX_WARPS);
-    unsigned long long *cnt = (unsigned long long *)(wcnt + MAX_WARPS * CNT_N);
+    unsigned long long *cnt = (unsigned long long *)(wcnt + MAX_WARPS * CNT_ROW);
     unsigned long long *ledger = cnt + CNT_N;
     unsigned long long *mbar = ledger + 3 * GPUMCD_MAX_PLANS_PER_RUN;
     CtaFlags *flags = (CtaFlags *)(mbar + 1);
@@ -1097,7 +1105,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
         ws[i].p_lo[0] = ws[i].p_hi[0] = ws[i].p_lo[1] = ws[i].p_hi[1] = 0;
         ws[i].q_lo[0] = ws[i].q_hi[0] = ws[i].q_lo[1] = ws[i].q_hi[1] = 0;
     }
-    for (int i = tid; i < MAX_WARPS * CNT_N; i += blockDim.x) wcnt[i] = 0u;
+    for (int i = tid; i < MAX_WARPS * CNT_ROW; i += blockDim.x) wcnt[i] = 0u;
     for (int i = tid; i < CNT_N + 3 * GPUMCD_MAX_PLANS_PER_RUN; i += blockDim.x) cnt[i] = 0;
     if (tid < 2) {
         flags->in_done[tid] = A.in_count[tid] == 0;
@@ -1263,7 +1271,8 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
     __syncthreads();
     for (int i = tid; i < CNT_N; i += blockDim.x) {
         unsigned long long n = cnt[i];
-        for (int k = 0; k < MAX_WARPS; ++k) n += wcnt[k * CNT_N + i];
+        if (row_word(i) < CNT_ROW)  // the cycle profile has no row
+            for (int k = 0; k < MAX_WARPS; ++k) n += wcnt[k * CNT_ROW + row_word(i)];
         if (n) atomicAdd(&A.counters[i], n);
     }
     for (int i = tid; i < 3 * A.n_plans; i += blockDim.x)
