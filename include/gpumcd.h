@@ -423,7 +423,10 @@ gpumcd_status gpumcd_debug_sample(gpumcd_ctx *ctx, int32_t kind, double p0, int3
  * events, Moller, bremsstrahlung, photons, electrons, overflows, spilled
  * particles, capped samplers, then cycles[2], passes[2] and active lanes[2]
  * of the photon and electron warps' event passes, refill cycles, type
- * switches). */
+ * switches).  A photon pass is up to four Woodcock flights and the
+ * interactions they end on, an electron pass one step (its active lanes sum to
+ * the electron steps).  The profile is of the kernel that serves any number of
+ * plans, also where the launch holds one. */
 gpumcd_status gpumcd_debug_counters(gpumcd_ctx *ctx, uint64_t *out, int32_t *count);
 
 /* A phantom's majorant tables (GPUMCD §II.A mu_max, §II.B.3 electron

@@ -440,7 +440,8 @@ class Context:
 
     def profile(self) -> dict:
         """Per-particle-type cycle profile of the last run (needs LAUNCH_PROFILE):
-        warp-cycles of the event passes, passes, lane occupancy, refill cycles."""
+        warp-cycles of the event passes, passes (up to four photon flights with
+        their interactions, or one electron step), lane occupancy, refill cycles."""
         c = self.debug_counters().astype(np.float64)
         base = 15
         cyc, it, lanes = c[base:base + 2], c[base + 2:base + 4], c[base + 4:base + 6]

@@ -157,9 +157,10 @@ enum {
     CNT_E_STEPS, CNT_HARD_REAL, CNT_HARD_FICT, CNT_MOLLER, CNT_BREM,
     CNT_PHOTONS, CNT_ELECTRONS, CNT_OVERFLOW, CNT_SPILLS, CNT_SAMPLER_CAP,
     // profile counters (GPUMCD_LAUNCH_PROFILE), per particle type (photon,
-    // electron): SM clock cycles of the warps' event passes, the passes, and
-    // the active lanes summed over them; then cycles in refills and the number
-    // of type switches
+    // electron): SM clock cycles of the warps' event passes, the passes (a
+    // photon pass is up to four flights and the interactions they end on, an
+    // electron pass one step), and the active lanes summed over them; then
+    // cycles in refills and the number of type switches
     CNT_PROF_CYC, CNT_PROF_ITER = CNT_PROF_CYC + NT, CNT_PROF_LANES = CNT_PROF_ITER + NT,
     CNT_PROF_REFILL_CYC = CNT_PROF_LANES + NT, CNT_PROF_SWITCHES,
     // converged passes over parked hard-event candidates (always counted)

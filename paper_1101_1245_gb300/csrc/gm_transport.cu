@@ -1245,6 +1245,13 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
 #pragma unroll 1
             for (int k = 1;; ++k) {
                 uint32_t dep_idx = 0, dep_e = 0;
+                if (prof) {  // each step is a pass of its own in the profile
+                    const unsigned stepm = __ballot_sync(FULL, p.act);
+                    if (lane == 0) {
+                        atomicAdd(&S.cnt[CNT_PROF_ITER + 1], 1ull);
+                        atomicAdd(&S.cnt[CNT_PROF_LANES + 1], (unsigned long long)__popc(stepm));
+                    }
+                }
                 if (p.act) {
                     count(S, w, CNT_E_STEPS);
                     electron_step<ONE>(A, S, p, gw, w, dep_idx, dep_e, fin);
@@ -1263,8 +1270,10 @@ __global__ void __launch_bounds__(MAXT, MINB) k_transport(const __grid_constant_
             __syncwarp();
             if (lane == 0) {
                 atomicAdd(&S.cnt[CNT_PROF_CYC + t], (unsigned long long)(clock64() - c0));
-                atomicAdd(&S.cnt[CNT_PROF_ITER + t], 1ull);
-                atomicAdd(&S.cnt[CNT_PROF_LANES + t], (unsigned long long)n_act);
+                if (t == 0) {
+                    atomicAdd(&S.cnt[CNT_PROF_ITER], 1ull);
+                    atomicAdd(&S.cnt[CNT_PROF_LANES], (unsigned long long)n_act);
+                }
             }
         }
     }
