@@ -967,8 +967,10 @@ def run_ablation(args):
     paper's second geometry with its timing beams: the lane refill policies of
     the persistent kernel.  base = a warp's lanes refill only when all are
     empty; comp N = every N-th pass (the paper's compaction after N steps);
-    pool = every pass (the production policy).  Tallies are identical under
-    every policy, which the line checks."""
+    pool = every pass.  These run one kernel, with one electron step a pass, and
+    differ in the refill alone; production = the default launch, which refills
+    at every pass too but takes up to four electron steps in it.  Tallies are
+    identical under every policy, which the line checks."""
     import hashlib
 
     import torch
@@ -977,7 +979,8 @@ def run_ablation(args):
     import workloads as W
 
     ctx = g.engine(0)
-    policies = [("base", g.REFILL_WHEN_EMPTY), ("comp64", 64), ("comp16", 16), ("comp4", 4), ("pool", 1)]
+    policies = [("base", g.REFILL_WHEN_EMPTY), ("comp64", 64), ("comp16", 16), ("comp4", 4),
+                ("pool", g.REFILL_EVERY_PASS), ("production", 1)]
     ev = (torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True))
     rows = []
     for particle in (W.ELECTRON, W.PHOTON):
@@ -1015,6 +1018,7 @@ def run_ablation(args):
                      "step_ms": {k: v[0] for k, v in times.items()},
                      "a_comp": {k: tb / times[k][1] for k in ("comp64", "comp16", "comp4")},
                      "a_pool": tb / times["pool"][1],
+                     "a_production": tb / times["production"][1],
                      "tallies_identical": len(hashes) == 1,
                      "paper_gtx480": PAPER_DIVRED[name]})
         ctx.plan_close(plan)

@@ -140,17 +140,22 @@ typedef struct {
 } gpumcd_launch;
 
 /* refill_period: 1 (the default) refills a warp's empty lanes at every pass,
- * the persistent "pool" of GPUMCD §II.C.3.  N >= 2 refills them only every
+ * like the persistent "pool" of GPUMCD §II.C.3; its passes are up to four
+ * photon flights, or up to four electron steps while three quarters of the
+ * lanes are stepping.  The other forms compare refill policies with each
+ * other: in them an electron pass is one step.  N >= 2 refills only every
  * N-th pass of the warp or when all its lanes are empty, like the paper's
  * stream compaction after N steps.  GPUMCD_REFILL_WHEN_EMPTY refills only
  * an empty warp, so each set of 32 particles runs until its slowest one ends
- * (the paper's base configuration).  In the last two forms a warp also
+ * (the paper's base configuration).  GPUMCD_REFILL_EVERY_PASS refills at every
+ * pass, the pool by itself.  With N >= 2 and GPUMCD_REFILL_WHEN_EMPTY a warp also
  * considers a low-occupancy type switch only on refill passes.  Hard-event
  * passes and type switches by stack level stay on in every form.  The
  * tallies do not depend on the form.  A form other than 1 runs a separately
  * compiled kernel: it needs none of GPUMCD_LAUNCH_PROFILE,
  * GPUMCD_LAUNCH_WARP_AGGREGATE or GPUMCD_LAUNCH_KERMA (else GPUMCD_ERR_INVALID_ARG). */
 #define GPUMCD_REFILL_WHEN_EMPTY 0xFFFFFFFFu
+#define GPUMCD_REFILL_EVERY_PASS 0xFFFFFFFEu
 
 #define GPUMCD_LAUNCH_WARP_AGGREGATE 1u /* combine a warp's deposits to one voxel into one atomic */
 #define GPUMCD_LAUNCH_PROFILE 2u        /* count clock cycles per event type (see gpumcd_debug_counters) */

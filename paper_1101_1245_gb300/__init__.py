@@ -31,8 +31,10 @@ LAUNCH_WARP_AGGREGATE = 1
 LAUNCH_PROFILE = 2
 LAUNCH_GRAPH = 4
 LAUNCH_KERMA = 8
-# refill_period of the launch: refill empty lanes only when the whole warp is empty
+# refill_period of the launch: refill empty lanes only when the whole warp is empty,
+# or at every pass with one electron step a pass (the refill policies compared)
 REFILL_WHEN_EMPTY = 0xFFFFFFFF
+REFILL_EVERY_PASS = 0xFFFFFFFE
 PARTICLE_TYPES = ("photon", "electron")
 
 STATUS = {

@@ -144,7 +144,7 @@ struct TransportArgs {
     HardRec *hard;                     // [warp][HARD_CAP] parked hard-event candidates
     uint32_t stack_cap, switch_high, refill_low, chunk;
     uint32_t flags;
-    uint32_t refill_period;            // 1: refill every pass; N: every N-th pass or when empty
+    uint32_t refill_period;            // see gpumcd.h
     uint32_t phsp;                     // a plan of the launch has a phase-space source
     uint2 round_key[10];               // one plan in the launch: its Philox round keys
     uint32_t tab_bytes;                // bytes of tables staged into shared memory (the loaded materials')
