@@ -171,6 +171,14 @@ enum {
 // Philox4x32-10 (Salmon et al., SC'11): 10 rounds of the two 32x32->64
 // multiplies with the Weyl-sequence key schedule.
 // ---------------------------------------------------------------------------
+__host__ __device__ __forceinline__ uint32_t mulhi(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (uint32_t)((uint64_t)a * b >> 32);
+#endif
+}
+
 __host__ __device__ __forceinline__ uint2 philox_round_key(uint2 k, int r) {
     return make_uint2(k.x + (uint32_t)r * 0x9E3779B9u, k.y + (uint32_t)r * 0xBB67AE85u);
 }
@@ -181,14 +189,8 @@ __host__ __device__ __forceinline__ uint4 philox4x32_10_keyed(uint4 c, const Rou
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
         const uint2 k = key(r);
-#ifdef __CUDA_ARCH__
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
-#else
-        const uint64_t p0 = 0xD2511F53ull * c.x, p1 = 0xCD9E8D57ull * c.z;
-        const uint32_t hi0 = (uint32_t)(p0 >> 32), lo0 = (uint32_t)p0;
-        const uint32_t hi1 = (uint32_t)(p1 >> 32), lo1 = (uint32_t)p1;
-#endif
+        const uint32_t hi0 = mulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
+        const uint32_t hi1 = mulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
         c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
     }
     return c;
@@ -208,28 +210,28 @@ struct PhiloxLineage {
 constexpr uint32_t kM0Inverse = 0x991A7CDBu, kM1Inverse = 0x6D7CAE67u;  // modulo 2^32
 static_assert(kM0Inverse * 0xD2511F53u == 1u && kM1Inverse * 0xCD9E8D57u == 1u, "inverses");
 
-__device__ __forceinline__ PhiloxLineage philox_lineage(uint32_t lo, uint32_t hi, uint2 k0, uint2 k1) {
-    const uint32_t x = __umulhi(0xCD9E8D57u, hi) ^ lo ^ k0.x;
-    return {0xCD9E8D57u * hi ^ k1.x, __umulhi(0xD2511F53u, x) ^ k1.y, 0xD2511F53u * x};
+__host__ __device__ __forceinline__ PhiloxLineage philox_lineage(uint32_t lo, uint32_t hi, uint2 k0, uint2 k1) {
+    const uint32_t x = mulhi(0xCD9E8D57u, hi) ^ lo ^ k0.x;
+    return {0xCD9E8D57u * hi ^ k1.x, mulhi(0xD2511F53u, x) ^ k1.y, 0xD2511F53u * x};
 }
-__device__ __forceinline__ uint32_t philox_lineage_b(uint32_t c, uint2 k1) {
-    return __umulhi(0xD2511F53u, c * kM0Inverse) ^ k1.y;
+__host__ __device__ __forceinline__ uint32_t philox_lineage_b(uint32_t c, uint2 k1) {
+    return mulhi(0xD2511F53u, c * kM0Inverse) ^ k1.y;
 }
-__device__ __forceinline__ uint2 philox_lineage_words(uint32_t a, uint32_t c, uint2 k0, uint2 k1) {
+__host__ __device__ __forceinline__ uint2 philox_lineage_words(uint32_t a, uint32_t c, uint2 k0, uint2 k1) {
     const uint32_t hi = (a ^ k1.x) * kM1Inverse;
-    return make_uint2((c * kM0Inverse) ^ __umulhi(0xCD9E8D57u, hi) ^ k0.x, hi);
+    return make_uint2((c * kM0Inverse) ^ mulhi(0xCD9E8D57u, hi) ^ k0.x, hi);
 }
 
 template <class RoundKey>
-__device__ __forceinline__ uint4 philox4x32_10_lineage(uint32_t draw, uint32_t hist, const PhiloxLineage &l,
-                                                       const RoundKey &key) {
-    const uint32_t z = __umulhi(0xD2511F53u, draw) ^ hist ^ key(0).y;
-    uint4 c = make_uint4(__umulhi(0xCD9E8D57u, z) ^ l.a, 0xCD9E8D57u * z, l.b ^ (0xD2511F53u * draw), l.c);
+__host__ __device__ __forceinline__ uint4 philox4x32_10_lineage(uint32_t draw, uint32_t hist,
+                                                                const PhiloxLineage &l, const RoundKey &key) {
+    const uint32_t z = mulhi(0xD2511F53u, draw) ^ hist ^ key(0).y;
+    uint4 c = make_uint4(mulhi(0xCD9E8D57u, z) ^ l.a, 0xCD9E8D57u * z, l.b ^ (0xD2511F53u * draw), l.c);
 #pragma unroll
     for (int r = 2; r < 10; ++r) {
         const uint2 k = key(r);
-        const uint32_t hi0 = __umulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
-        const uint32_t hi1 = __umulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
+        const uint32_t hi0 = mulhi(0xD2511F53u, c.x), lo0 = 0xD2511F53u * c.x;
+        const uint32_t hi1 = mulhi(0xCD9E8D57u, c.z), lo1 = 0xCD9E8D57u * c.z;
         c = make_uint4(hi1 ^ c.y ^ k.x, lo1, hi0 ^ c.w ^ k.y, lo0);
     }
     return c;
