@@ -94,7 +94,8 @@ __device__ __forceinline__ float interp_ms(const float *t, float x) {
 // ors in the kernel's arguments.  A draw's ten rounds are about a quarter of
 // the transport's time (a build with six is 9-11% faster).  ONE takes 1e6 15
 // MeV electrons on 128^3 water from 1.77 to 1.74 ms, 4e6 photons from 4.10 to
-// 4.00 ms, 4e6 photons on the slabs from 3.12 to 3.05 ms, and needs no spills.
+// 4.00 ms, 4e6 photons on the slabs from 3.12 to 3.05 ms, and spills less (4
+// bytes a thread are loaded back instead of 12).
 // Only the keys are read there: with the plan's other fields in the arguments
 // too, the compiler contracts other multiply-adds (the tallies move) and the
 // beams above take 0.4% more to 1.8% less than without ONE.

@@ -5,26 +5,27 @@ instruction issue of the SMs (FP32/INT ALU work, divergence and latency).  The
 ceiling is 4 warp-instructions per clock per SM (one per SM sub-partition),
 times the SM count and the SM clock sampled during the timed region.
 
-The algorithmic work of one launch is counted in warp-instructions that a
-fully converged warp would issue: the per-unit costs below times the transport
-events (electron condensed-history steps plus photon Woodcock events) that the
-kernel itself counts.  The per-unit costs come from ncu on the same workload
-at reduced history counts (smsp__inst_executed.sum x
-smsp__thread_inst_executed_per_inst_executed.ratio / 32, divided by the
-kernel's event counts), separately for the electron and the photon beam
-because their mixes of step and event types differ.
+The work of one launch is counted in warp-instructions that a fully converged
+warp would issue: the per-unit costs below times the transport events (electron
+condensed-history steps plus photon Woodcock events) that the kernel itself
+counts.  The per-unit costs are those of the present kernel, from ncu on the same
+workload at reduced history counts (smsp__thread_inst_executed.sum / 32, divided
+by the kernel's event counts), separately for the electron and the photon beam
+because their mixes of step and event types differ; they are measured again when
+the kernel's instructions change.  So the fraction is the issue slots used times
+the lanes filled in them, and says nothing about how few instructions an event
+could do with.
 """
 from __future__ import annotations
 
 from typing import Optional
 
-# converged warp-instructions per transport event, electron beam / photon beam: the
-# physics of a step or photon event, measured on the kernel that ran each hard event
-# inline (no parking).  The kernel that parks hard-event candidates for converged
-# passes executes 22.8 / 20.4 per event (the parking is scheduling, not physics), so
-# these are the algorithmic figures
-INST_PER_EVENT_E_BEAM: Optional[float] = 19.68
-INST_PER_EVENT_PH_BEAM: Optional[float] = 18.81
+# converged warp-instructions per transport event, electron beam / photon beam of the
+# timing workload (launches of one plan) at a fifth of its histories: 8.364e9
+# thread-instructions over 15.73e6 events, and 17.377e9 over 36.11e6
+# (bench.py --ncu-case --workload c2)
+INST_PER_EVENT_E_BEAM: Optional[float] = 16.62
+INST_PER_EVENT_PH_BEAM: Optional[float] = 15.04
 # DRAM bytes (read + write) per transport launch of the timing workload: measured with
 # 32 batch tallies (2.87e9 per launch); the benchmark now runs it with 16, whose tally
 # traffic that capture does not describe, so None until it is captured again
@@ -53,19 +54,14 @@ def alu_roofline(events_e_beam: int, events_ph_beam: int, kernel_ms: float, sm_m
 # per transport event (smsp__thread_inst_executed.sum / 32 / events) in the
 # electron-beam and the photon-beam launch sequences, from ncu on the
 # workload's 27 plans of at most 160^3 voxels at 1/10 of their first round
-# (bench.py --ncu-case --workload c4): 144.79e9 thread-instructions over
-# 259.66e6 events, and 72.61e9 over 128.58e6.  Kept fixed as the algorithmic
-# work per event, so a faster kernel shows as a higher achieved rate.
-INST_PER_EVENT_C4_E_SEQ: Optional[float] = 17.43
-INST_PER_EVENT_C4_PH_SEQ: Optional[float] = 17.65
-# DRAM bytes (read + write) per event of the same case on the current kernel (one
-# 1024-thread CTA per SM, tables packed per material, a photon's majorant taken once
-# per pass, each electron step's majorant from its own voxel, event-path divisions as
-# reciprocal-multiply, the step's draw taken while its voxel word loads, the inside
-# and cut-off tests of primaries at their claim): 1.907 GB over 247.16e6 events
-# (electron sequence) and 1.817 GB over 124.71e6 (photon sequence)
-TRAFFIC_BYTES_PER_EVENT_C4_E_SEQ: Optional[float] = 7.71
-TRAFFIC_BYTES_PER_EVENT_C4_PH_SEQ: Optional[float] = 14.57
+# (bench.py --ncu-case --workload c4): 105.81e9 thread-instructions over
+# 247.16e6 events, and 54.76e9 over 124.71e6.
+INST_PER_EVENT_C4_E_SEQ: Optional[float] = 13.38
+INST_PER_EVENT_C4_PH_SEQ: Optional[float] = 13.72
+# DRAM bytes (read + write) per event of the same case: 1.893 GB (electron
+# sequence) and 1.790 GB (photon sequence)
+TRAFFIC_BYTES_PER_EVENT_C4_E_SEQ: Optional[float] = 7.66
+TRAFFIC_BYTES_PER_EVENT_C4_PH_SEQ: Optional[float] = 14.35
 
 
 def alu_roofline_c4(events_e_seq: int, events_ph_seq: int, kernel_ms: float, sm_mhz: Optional[float],
