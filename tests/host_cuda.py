@@ -14,11 +14,12 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 
 @functools.lru_cache(None)
 def library() -> C.CDLL:
-    out = os.path.join(tempfile.mkdtemp(), "host_cuda.so")
-    subprocess.run([b.nvcc(), "-std=c++17", "-O1", *b.ARCH, "-Xcompiler", "-fPIC", "-I", b.INCLUDE, "-I", b.CSRC,
-                    "-x", "cu", "-shared", "-cudart", "none", "-Xlinker", "-Bsymbolic", "-o", out, os.path.join(b.CSRC, "gm_api.cu"),
-                    os.path.join(HERE, "host_cuda.cpp")], check=True)
-    L = C.CDLL(out)
+    with tempfile.TemporaryDirectory() as d:
+        out = os.path.join(d, "host_cuda.so")
+        subprocess.run([b.nvcc(), "-std=c++17", "-O1", *b.ARCH, "-Xcompiler", "-fPIC", "-I", b.INCLUDE, "-I", b.CSRC,
+                        "-x", "cu", "-shared", "-cudart", "none", "-Xlinker", "-Bsymbolic", "-o", out,
+                        os.path.join(b.CSRC, "gm_api.cu"), os.path.join(HERE, "host_cuda.cpp")], check=True)
+        L = C.CDLL(out)
     for name, (res, args) in g.SIGNATURES.items():
         f = getattr(L, name)
         f.restype, f.argtypes = res, args
